@@ -272,11 +272,11 @@ LBM_API const char *lbm_last_error(const lbm_ctx *ctx);
  * fused pass on even and odd steps (0..LBM_COLLIDE_CONFIGS-1): thread-block
  * shape and register budget; fused shape 4 stores with the streaming cache
  * policy; fused shapes 5-9 walk runs of planes per block and copy the next
- * plane's populations (shapes 8-9: and the neighbour densities) into shared
- * memory while colliding the current one (shape 9: with streaming stores).
- * A new context starts with the shapes measured fastest for its storage on
- * a 256^3 lattice (float32 1/6/7, half and bfloat16 offsets 0/6/8, local
- * offsets 0/9/9).  Results do not depend on the choice; speed does (the
+ * plane's populations (shapes 5, 8, 9: and the neighbour densities) into shared
+ * memory while colliding the current one (shapes 5, 9: with streaming
+ * stores).  A new context starts with the shapes measured fastest for its
+ * storage on a 256^3 lattice (float32 1/6/7, half and bfloat16 offsets 0/9/8,
+ * local offsets 0/9/9).  Results do not depend on the choice; speed does (the
  * autotuner measures them per lattice size and storage).  EINVAL if out of
  * range. */
 #define LBM_DENSITY_CONFIGS 3

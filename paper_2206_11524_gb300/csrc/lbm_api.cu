@@ -197,7 +197,8 @@ float stored_ref(const lbm_ctx *c, const float *rho_enc_host, int s, int i,
                  int x, int y, int z) {
   if (hmcsc::storage_local(c->sp.storage))
     return hmcsc::wgt(i) * rho_enc_host[2 * tiled_node(c, x, y, z) + s];
-  return c->sp.ref[s][hmcsc::wclass(i)];
+  const float2 r = c->sp.ref[hmcsc::wclass(i)];
+  return s == 0 ? r.x : r.y;
 }
 
 // Index (in stored values) of population (component s, direction i) = slot
@@ -342,11 +343,13 @@ lbm_status lbm_create(const lbm_params *params, void *d_workspace,
   }
   sp.G = (float)params->G;
   sp.storage = params->storage;
-  for (int s = 0; s < 2; ++s) {
-    const float r0 = (float)params->rho0[s];
-    sp.ref[s][0] = hmcsc::wgt(0) * r0;
-    sp.ref[s][1] = hmcsc::wgt(1) * r0;
-    sp.ref[s][2] = hmcsc::wgt(4) * r0;
+  const float r0[2] = {(float)params->rho0[0], (float)params->rho0[1]};
+  const float scale = params->storage == LBM_STORAGE_F16_OFFSET ? hmcsc::kHalfScale : 1.0f;
+  const int dir_of_class[3] = {0, 1, 4};
+  for (int k = 0; k < 3; ++k) {
+    const float w = hmcsc::wgt(dir_of_class[k]);
+    sp.ref[k] = make_float2(w * r0[0], w * r0[1]);
+    sp.nref[k] = make_float2(sp.ref[k].x * -scale, sp.ref[k].y * -scale);
   }
   for (int d = 0; d < 3; ++d) sp.F[d] = (float)params->F_ext[d];
   memset(&sp.res, 0, sizeof sp.res);
@@ -365,8 +368,8 @@ lbm_status lbm_create(const lbm_params *params, void *d_workspace,
   const bool local = hmcsc::storage_local(params->storage);
   const bool f32 = params->storage == LBM_STORAGE_F32;
   c->launch_cfg[0] = f32 ? 1 : 0;
-  c->launch_cfg[1] = local ? 9 : 6;
-  c->launch_cfg[2] = local ? 9 : (f32 ? 7 : 8);
+  c->launch_cfg[1] = f32 ? 6 : 9;
+  c->launch_cfg[2] = f32 ? 7 : local ? 9 : 8;
   c->single_pass_zc = 0;
   c->wave_cfg = 0;
   c->wave_lag = hmcsc::kWaveLagDefault;

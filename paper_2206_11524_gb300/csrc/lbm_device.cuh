@@ -89,15 +89,14 @@ __device__ __forceinline__ float2 dec_ref(const StepParams &p, float2 own_prev,
                                           int i) {
   if (storage_local(ST))
     return make_float2(__fmul_rn(wgt(i), own_prev.x), __fmul_rn(wgt(i), own_prev.y));
-  return make_float2(p.ref[0][wclass(i)], p.ref[1][wclass(i)]);
+  return p.ref[wclass(i)];
 }
 
 // The 19 populations of both components at the current time step, decoded
 // to float32.
 template <int PARITY, int ST>
 __device__ __forceinline__ void load_pops(const StepParams &p, const Workspace &w,
-                                          const Geo &g, float (&v1)[kQ],
-                                          float (&v2)[kQ]) {
+                                          const Geo &g, float2 (&v)[kQ]) {
   using C = Codec2<ST>;
   const typename C::T2 *f = static_cast<const typename C::T2 *>(w.f);
   const long long nodes = p.ntiles * kTile, pairs = p.ntiles * kTilePairs;
@@ -115,29 +114,26 @@ __device__ __forceinline__ void load_pops(const StepParams &p, const Workspace &
     if (kChecked && !in_bounds(w.fault, (src - f) + slot * kTile, pairs, kFaultPopLoad))
       src = f - slot * kTile;  // reads element 0
     const typename C::T2 raw = src[slot * kTile];
-    const float2 v = C::dec(raw, dec_ref<ST>(p, own_prev, i));
-    v1[i] = v.x;
-    v2[i] = v.y;
+    v[i] = C::dec(raw, dec_ref<ST>(p, own_prev, i));
   }
 }
 
-// Zeroth moment, summed in direction order; k_density and k_collide_stream
-// share this order so both see bit-identical densities.
-__device__ __forceinline__ float sum19(const float (&v)[kQ]) {
-  float r = v[0];
+// Zeroth moment of both components, summed in direction order; k_density
+// and k_collide_stream share this order so both see bit-identical densities.
+__device__ __forceinline__ float2 sum19(const float2 (&v)[kQ]) {
+  float2 r = v[0];
 #pragma unroll
-  for (int i = 1; i < kQ; ++i) r += v[i];
+  for (int i = 1; i < kQ; ++i) r = add2(r, v[i]);
   return r;
 }
 
-__device__ __forceinline__ void first_moment(const float (&v)[kQ],
-                                             float (&j)[3]) {
-  j[0] = j[1] = j[2] = 0.0f;
+__device__ __forceinline__ void first_moment(const float2 (&v)[kQ], float2 (&j)[3]) {
+  j[0] = j[1] = j[2] = pair_of(0.0f);
 #pragma unroll
   for (int i = 1; i < kQ; ++i) {
-    if (cx(i)) j[0] += cx(i) > 0 ? v[i] : -v[i];
-    if (cy(i)) j[1] += cy(i) > 0 ? v[i] : -v[i];
-    if (cz(i)) j[2] += cz(i) > 0 ? v[i] : -v[i];
+    if (cx(i)) j[0] = cx(i) > 0 ? add2(j[0], v[i]) : sub2(j[0], v[i]);
+    if (cy(i)) j[1] = cy(i) > 0 ? add2(j[1], v[i]) : sub2(j[1], v[i]);
+    if (cz(i)) j[2] = cz(i) > 0 ? add2(j[2], v[i]) : sub2(j[2], v[i]);
   }
 }
 
@@ -195,35 +191,44 @@ __device__ __forceinline__ GlobalRho global_rho(const StepParams &p, const Works
 // a_sigma(x + c_i) c_i, a_sigma = G_ads,2 n_s,sigma (G_ads,1 = -G_ads,2,
 // Table 1; the indicator of Eq. 4 is the component's own fraction).  With
 // one fraction for both (PC = false) A_1 = A_2.  Opposite directions are
-// summed as pairs, so a uniform field gives exactly zero.
+// summed as pairs, so a uniform field gives exactly zero.  Every product is
+// fused into the sum it enters, written out so that each kernel rounds alike.
+// gf[d] = (g_1, g_2) along axis d.
 template <bool PC, typename RS>
 __device__ __forceinline__ void force_per_mass(const StepParams &p, const RS &rs,
-                                               const Workspace &w, const Geo &g,
-                                               float rho_tot, float (&g1)[3],
-                                               float (&g2)[3]) {
-  float s1[3] = {0.f, 0.f, 0.f}, s2[3] = {0.f, 0.f, 0.f};
-  float sa[3] = {0.f, 0.f, 0.f}, sb[3] = {0.f, 0.f, 0.f};
+                                               float rho_tot, float2 (&gf)[3]) {
+  float2 s[3], sab[3];  // (S_1, S_2) and (A_1, A_2), the latter when PC
+  float sa[3];          // A otherwise
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    s[d] = sab[d] = pair_of(0.0f);
+    sa[d] = 0.0f;
+  }
 #pragma unroll
   for (int i = 1; i <= 9; ++i) {
-    const float2 rp = rs.at(cx(i), cy(i), cz(i));
-    const float2 rm = rs.at(-cx(i), -cy(i), -cz(i));
-    const float ap = rs.a1(cx(i), cy(i), cz(i));
-    const float am = rs.a1(-cx(i), -cy(i), -cz(i));
-    const float d1 = wgt(i) * (rp.x - rm.x);
-    const float d2 = wgt(i) * (rp.y - rm.y);
-    const float da = wgt(i) * (ap - am);
-    float db = 0.0f;
-    if (PC) db = wgt(i) * (rs.a2(cx(i), cy(i), cz(i)) - rs.a2(-cx(i), -cy(i), -cz(i)));
-    if (cx(i)) { s1[0] += cx(i) > 0 ? d1 : -d1; s2[0] += cx(i) > 0 ? d2 : -d2; sa[0] += cx(i) > 0 ? da : -da; if (PC) sb[0] += cx(i) > 0 ? db : -db; }
-    if (cy(i)) { s1[1] += cy(i) > 0 ? d1 : -d1; s2[1] += cy(i) > 0 ? d2 : -d2; sa[1] += cy(i) > 0 ? da : -da; if (PC) sb[1] += cy(i) > 0 ? db : -db; }
-    if (cz(i)) { s1[2] += cz(i) > 0 ? d1 : -d1; s2[2] += cz(i) > 0 ? d2 : -d2; sa[2] += cz(i) > 0 ? da : -da; if (PC) sb[2] += cz(i) > 0 ? db : -db; }
+    const float2 dr = sub2(rs.at(cx(i), cy(i), cz(i)), rs.at(-cx(i), -cy(i), -cz(i)));
+    const float da1 = __fsub_rn(rs.a1(cx(i), cy(i), cz(i)), rs.a1(-cx(i), -cy(i), -cz(i)));
+    float2 da = pair_of(0.0f);
+    if (PC) da = make_float2(da1, __fsub_rn(rs.a2(cx(i), cy(i), cz(i)),
+                                            rs.a2(-cx(i), -cy(i), -cz(i))));
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int c = d == 0 ? cx(i) : d == 1 ? cy(i) : cz(i);
+      if (c == 0) continue;
+      const float w = c > 0 ? wgt(i) : -wgt(i);
+      s[d] = fma2(pair_of(w), dr, s[d]);
+      if (PC)
+        sab[d] = fma2(pair_of(w), da, sab[d]);
+      else
+        sa[d] = __fmaf_rn(w, da1, sa[d]);
+    }
   }
   const float inv_rho = 1.0f / rho_tot;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    const float fe = p.F[d] * inv_rho;
-    g1[d] = -p.G * s2[d] + sa[d] + fe;
-    g2[d] = -p.G * s1[d] - (PC ? sb[d] : sa[d]) + fe;
+    const float a1 = PC ? sab[d].x : sa[d], a2 = PC ? sab[d].y : sa[d];
+    gf[d].x = __fmaf_rn(p.F[d], inv_rho, __fmaf_rn(-p.G, s[d].y, a1));
+    gf[d].y = __fmaf_rn(p.F[d], inv_rho, __fmaf_rn(-p.G, s[d].x, -a2));
   }
 }
 
@@ -273,8 +278,7 @@ __device__ __forceinline__ float res_u(const StepParams &p, int face, int d) {
 // density reservoir, at the face's velocity for velocity boundary cells.
 // Only blocks whose box meets a reservoir (`maybe`, block-uniform) look.
 __device__ __forceinline__ void reservoir_state(const StepParams &p, bool maybe,
-                                                int x, int y, int z,
-                                                float (&v1)[kQ], float (&v2)[kQ]) {
+                                                int x, int y, int z, float2 (&v)[kQ]) {
   if (!maybe) return;
   const int face = res_face(p, x, y, z);
   if (face >= 0) {
@@ -282,16 +286,11 @@ __device__ __forceinline__ void reservoir_state(const StepParams &p, bool maybe,
     if (p.res.moving) {
       const float ux = res_u(p, face, 0), uy = res_u(p, face, 1), uz = res_u(p, face, 2);
 #pragma unroll
-      for (int i = 0; i < kQ; ++i) {
-        v1[i] = res_feq(i, r1, ux, uy, uz);
-        v2[i] = res_feq(i, r2, ux, uy, uz);
-      }
+      for (int i = 0; i < kQ; ++i)
+        v[i] = make_float2(res_feq(i, r1, ux, uy, uz), res_feq(i, r2, ux, uy, uz));
     } else {
 #pragma unroll
-      for (int i = 0; i < kQ; ++i) {
-        v1[i] = wgt(i) * r1;
-        v2[i] = wgt(i) * r2;
-      }
+      for (int i = 0; i < kQ; ++i) v[i] = make_float2(wgt(i) * r1, wgt(i) * r2);
     }
   }
 }
@@ -301,20 +300,17 @@ __device__ __forceinline__ void reservoir_state(const StepParams &p, bool maybe,
 // reference: w_i times the destination's density at this step (*_LOCAL;
 // rho_s for the rest population, the density pass's value otherwise), or the
 // constants w_i rho0_sigma (*_OFFSET).
-template <int PARITY, int ST, typename RS, bool CS = false>
+template <int PARITY, int ST, typename RS, bool CS = false, typename GE>
 __device__ __forceinline__ void put2(const StepParams &p, const Workspace &w,
-                                     const Geo &g, const RS &rs, int i, float o1,
-                                     float o2, float r1, float r2) {
+                                     const GE &g, const RS &rs, int i, float2 o,
+                                     float2 rho) {
   using C = Codec2<ST>;
   typename C::T2 *f = static_cast<typename C::T2 *>(w.f);
-  // encoding reference times the codec's scale (exact)
-  float2 ref = make_float2(p.ref[0][wclass(i)] * C::kScale, p.ref[1][wclass(i)] * C::kScale);
-  if (storage_local(ST)) {
-    const float2 rd = i == 0 ? make_float2(r1, r2) : rs.late(cx(i), cy(i), cz(i));
-    const float ws = wgt(i) * C::kScale;
-    ref = make_float2(__fmul_rn(ws, rd.x), __fmul_rn(ws, rd.y));
-  }
-  const typename C::T2 e = C::enc_s(o1, o2, ref);
+  typename C::T2 e;
+  if constexpr (storage_local(ST))
+    e = C::enc_local(o, wgt(i), i == 0 ? rho : rs.late(cx(i), cy(i), cz(i)));
+  else
+    e = C::enc(o, p.nref[wclass(i)]);
   const int slot = PARITY == 0 ? opp(i) : i;
   typename C::T2 *dst = f + (PARITY == 0 ? g.pop_off(0, 0, 0) : g.pop_off(cx(i), cy(i), cz(i)));
   if (!kChecked ||
@@ -335,105 +331,119 @@ __device__ __forceinline__ void put2(const StepParams &p, const Workspace &w,
 // step.  The relaxation weight b = (1 - n_s) / tau is folded into the
 // equilibrium: B_i = b f^eq_i = (b w_i rho_s)[1 - 1.5 u.u + 4.5 (c_i.u)^2
 // +- 3 c_i.u], so each population costs two fused multiply-adds on top of B_i.
+// Every value is the pair of both components.  With E_i = 1 - 1.5 u.u + 4.5
+// (c_i.u)^2 and q = 3 b w_i rho, the two products of B_i = b w_i rho E_i + q
+// c_i.u cannot both be fused: component 1 rounds q c_i.u and component 2
+// rounds b w_i rho E_i, the order every result of this library has been
+// computed in, so these six operations stay scalar.
 struct Relax {
-  float a, base, br, br18, br36, moving, nsx;
-  __device__ __forceinline__ Relax(float om, float ns_s, float rho_s, const float (&u)[3]) {
-    nsx = ns_s;
-    a = (1.0f - nsx) * (1.0f - om);
-    const float b = (1.0f - nsx) * om;
-    base = 1.0f - 1.5f * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-    br = b * rho_s;
-    br18 = br * (1.0f / 18.0f);
-    br36 = br * (1.0f / 36.0f);
-    moving = 0.0f;  // sum of B_i over the 18 moving directions
+  float2 a, base, br, br18, br36, q18, q36, moving, ns;
+  __device__ __forceinline__ Relax(float2 om, float2 ns_s, float2 rho, const float2 (&u)[3]) {
+    ns = ns_s;
+    const float2 open = sub2(pair_of(1.0f), ns);
+    a = mul2(open, sub2(pair_of(1.0f), om));
+    base = fma2(pair_of(-1.5f), fma2(u[2], u[2], fma2(u[0], u[0], mul2(u[1], u[1]))),
+                pair_of(1.0f));
+    br = mul2(mul2(open, om), rho);
+    br18 = mul2(br, pair_of(1.0f / 18.0f));
+    br36 = mul2(br, pair_of(1.0f / 36.0f));
+    q18 = mul2(pair_of(3.0f), br18);
+    q36 = mul2(pair_of(3.0f), br36);
+    moving = pair_of(0.0f);  // sum of B_i over the 18 moving directions
   }
-  // post-collision values of the opposite pair (i, i + 9) from their
-  // pre-collision values vi, vj
-  __device__ __forceinline__ void pair_s(int i, const float (&u)[3], float vi, float vj,
-                                         float &out_i, float &out_j) {
-    const float cu = cx(i) * u[0] + cy(i) * u[1] + cz(i) * u[2];
-    const float bw = wgt(i) == (1.0f / 18.0f) ? br18 : br36;
-    const float even = bw * fmaf(4.5f * cu, cu, base);
-    const float odd = (3.0f * bw) * cu;
-    const float B_i = even + odd, B_j = even - odd;
-    moving += B_i + B_j;
-    out_i = fmaf(a, vi, fmaf(nsx, vj, B_i));
-    out_j = fmaf(a, vj, fmaf(nsx, vi, B_j));
-  }
-  __device__ __forceinline__ void pair(int i, const float (&u)[3], const float (&v)[kQ],
-                                       float &out_i, float &out_j) {
-    pair_s(i, u, v[i], v[i + 9], out_i, out_j);
+  // post-collision values of the opposite pair of directions (i, j) from
+  // their pre-collision values vi, vj; cu = c_i . u
+  __device__ __forceinline__ void pair(bool axis, float2 cu, float2 vi, float2 vj,
+                                       float2 &out_i, float2 &out_j) {
+    const float2 bw = axis ? br18 : br36, q = axis ? q18 : q36;
+    const float2 e = fma2(mul2(pair_of(4.5f), cu), cu, base);
+    const float odd1 = __fmul_rn(q.x, cu.x), even2 = __fmul_rn(bw.y, e.y);
+    const float2 B_i = make_float2(__fmaf_rn(bw.x, e.x, odd1), __fmaf_rn(q.y, cu.y, even2));
+    const float2 B_j = make_float2(__fmaf_rn(bw.x, e.x, -odd1), __fmaf_rn(-q.y, cu.y, even2));
+    moving = add2(moving, add2(B_i, B_j));
+    out_i = fma2(a, vi, fma2(ns, vj, B_i));
+    out_j = fma2(a, vj, fma2(ns, vi, B_j));
   }
   // post-collision rest population: B_0 = b rho_s - sum of the moving B_i
-  __device__ __forceinline__ float rest_s(float v0) const {
-    return fmaf(a + nsx, v0, br - moving);
+  __device__ __forceinline__ float2 rest(float2 v0) const {
+    return fma2(make_float2(__fadd_rn(a.x, ns.x), __fadd_rn(a.y, ns.y)), v0, sub2(br, moving));
   }
-  __device__ __forceinline__ float rest(const float (&v)[kQ]) const { return rest_s(v[0]); }
 };
 
-template <int PARITY, int ST, typename RS, bool CS = false>
+template <int PARITY, int ST, typename RS, bool CS = false, typename GE>
 __device__ __forceinline__ void collide_put2(const StepParams &p, const Workspace &w,
-                                             const Geo &g, const RS &rs,
-                                             const float (&v1)[kQ],
-                                             const float (&v2)[kQ], float r1,
-                                             float r2, const float (&u1)[3],
-                                             const float (&u2)[3], float ns1,
-                                             float ns2) {
-  Relax c1(p.omega[0], ns1, r1, u1), c2(p.omega[1], ns2, r2, u2);
+                                             const GE &g, const RS &rs,
+                                             const float2 (&v)[kQ], float2 rho,
+                                             const float2 (&u)[3], float2 ns) {
+  Relax c(make_float2(p.omega[0], p.omega[1]), ns, rho, u);
 #pragma unroll
   for (int i = 1; i <= 9; ++i) {
-    float o1i, o1j, o2i, o2j;
-    c1.pair(i, u1, v1, o1i, o1j);
-    c2.pair(i, u2, v2, o2i, o2j);
-    put2<PARITY, ST, RS, CS>(p, w, g, rs, i, o1i, o2i, r1, r2);
-    put2<PARITY, ST, RS, CS>(p, w, g, rs, i + 9, o1j, o2j, r1, r2);
+    // of the two, j = i + 9 has the positive first nonzero component, so
+    // c_j . u starts without a negation
+    const int j = i + 9;
+    float2 cu = pair_of(0.0f);
+    bool first = true;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int c = d == 0 ? cx(j) : d == 1 ? cy(j) : cz(j);
+      if (c == 0) continue;
+      cu = first ? u[d] : (c > 0 ? add2(cu, u[d]) : sub2(cu, u[d]));
+      first = false;
+    }
+    float2 oi, oj;
+    c.pair(wclass(i) == 1, cu, v[j], v[i], oj, oi);
+    put2<PARITY, ST, RS, CS>(p, w, g, rs, i, oi, rho);
+    put2<PARITY, ST, RS, CS>(p, w, g, rs, j, oj, rho);
   }
-  put2<PARITY, ST, RS, CS>(p, w, g, rs, 0, c1.rest(v1), c2.rest(v2), r1, r2);
+  put2<PARITY, ST, RS, CS>(p, w, g, rs, 0, c.rest(v[0]), rho);
 }
 
-// Moments, forces, equilibrium velocity and collision of node (x, y, z)
-// given its neighbourhood g and the source of the step's densities.
-// collide_loaded starts from the node's 38 populations already decoded (and
-// replaced by the prescribed state inside a reservoir).
-template <int PARITY, int ST, bool PC, typename RS, bool CS = false>
+// Moments, forces, equilibrium velocity and collision of one node, given
+// where its neighbours' slots lie (g: pop_off) and where the step's densities
+// are found.  collide_loaded starts from the node's 19 pairs already decoded
+// (and replaced by the prescribed state inside a reservoir) and its n_s.
+template <int PARITY, int ST, bool PC, typename RS, bool CS = false, typename GE>
 __device__ __forceinline__ void collide_loaded(const StepParams &p, const Workspace &w,
-                                               const Geo &g, const RS &rs,
-                                               const float (&f1)[kQ],
-                                               const float (&f2)[kQ]) {
-  const float r1 = sum19(f1), r2 = sum19(f2);
-  float j1[3], j2[3];
-  first_moment(f1, j1);
-  first_moment(f2, j2);
+                                               const GE &g, const RS &rs,
+                                               const float2 (&v)[kQ], float2 ns) {
+  const float2 rho = sum19(v);
+  float2 j[3];
+  first_moment(v, j);
 
-  float g1[3], g2[3];
-  force_per_mass<PC>(p, rs, w, g, r1 + r2, g1, g2);
+  float2 gf[3];
+  force_per_mass<PC>(p, rs, __fadd_rn(rho.x, rho.y), gf);
 
   // Eq. 6: common velocity sum_s j_s/tau_s / sum_s rho_s/tau_s, then the
   // Shan-Chen shift tau_s F_tot,s / rho_s = tau_s g_s.
-  const float inv_den = 1.0f / (r1 * p.omega[0] + r2 * p.omega[1]);
-  float u1[3], u2[3];
+  const float inv_den = 1.0f / __fmaf_rn(rho.x, p.omega[0], __fmul_rn(rho.y, p.omega[1]));
+  float2 u[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    const float uc = (j1[d] * p.omega[0] + j2[d] * p.omega[1]) * inv_den;
-    u1[d] = uc + p.tau[0] * g1[d];
-    u2[d] = uc + p.tau[1] * g2[d];
+    const float jc = __fmaf_rn(j[d].x, p.omega[0], __fmul_rn(j[d].y, p.omega[1]));
+    u[d].x = __fmaf_rn(jc, inv_den, __fmul_rn(p.tau[0], gf[d].x));
+    u[d].y = __fmaf_rn(jc, inv_den, __fmul_rn(p.tau[1], gf[d].y));
   }
 
+  collide_put2<PARITY, ST, RS, CS>(p, w, g, rs, v, rho, u, ns);
+}
+
+// n_s,1 and n_s,2 (the same without per-component fractions) of a node.
+template <bool PC>
+__device__ __forceinline__ float2 node_ns(const StepParams &p, const Workspace &w, const Geo &g) {
   int own = g.node(0, 0, 0);
   if (!in_bounds(w.fault, own, p.ntiles * kTile, kFaultGeometry)) own = 0;
   const float ns1 = w.ns[own];
-  const float ns2 = PC ? w.ns2[own] : ns1;
-  collide_put2<PARITY, ST, RS, CS>(p, w, g, rs, f1, f2, r1, r2, u1, u2, ns1, ns2);
+  return make_float2(ns1, PC ? w.ns2[own] : ns1);
 }
 
 template <int PARITY, int ST, bool PC, typename RS>
 __device__ __forceinline__ void collide_node(const StepParams &p, const Workspace &w,
                                              const Geo &g, const RS &rs,
                                              bool maybe_res, int x, int y, int z) {
-  float f1[kQ], f2[kQ];
-  load_pops<PARITY, ST>(p, w, g, f1, f2);
-  reservoir_state(p, maybe_res, x, y, z, f1, f2);
-  collide_loaded<PARITY, ST, PC>(p, w, g, rs, f1, f2);
+  float2 v[kQ];
+  load_pops<PARITY, ST>(p, w, g, v);
+  reservoir_state(p, maybe_res, x, y, z, v);
+  collide_loaded<PARITY, ST, PC>(p, w, g, rs, v, node_ns<PC>(p, w, g));
 }
 
 template <int PARITY, int ST, bool PC, bool CS = false>
@@ -441,10 +451,11 @@ __device__ __forceinline__ void collide_body(const StepParams &p,
                                              const Workspace &w, bool maybe_res,
                                              int x, int y, int z) {
   const Geo g = make_geo(p, x, y, z);
-  float f1[kQ], f2[kQ];
-  load_pops<PARITY, ST>(p, w, g, f1, f2);
-  reservoir_state(p, maybe_res, x, y, z, f1, f2);
-  collide_loaded<PARITY, ST, PC, GlobalRho, CS>(p, w, g, global_rho(p, w, g), f1, f2);
+  float2 v[kQ];
+  load_pops<PARITY, ST>(p, w, g, v);
+  reservoir_state(p, maybe_res, x, y, z, v);
+  collide_loaded<PARITY, ST, PC, GlobalRho, CS>(p, w, g, global_rho(p, w, g), v,
+                                                node_ns<PC>(p, w, g));
 }
 
 
@@ -460,37 +471,30 @@ __host__ __device__ constexpr Shape density_shape(int cfg) {
   return cfg == 1 ? Shape{8, 1, 1} : cfg == 2 ? Shape{4, 1, 1} : Shape{4, 2, 1};
 }
 // Shapes of the prefetching fused pass (k_collide_pipe): block 32 x by,
-// blocks per SM, planes per block (zc) and shared-memory buffers (nb, so
-// nb - 1 planes are in flight).
+// blocks per SM.  On the 256^3 electrode (us, even / odd step; 168 and 176
+// bytes a node at the copy rate of 6690 GB/s are 421 and 441): half offsets
+// 559/633 in shape 6, 438/528 in shapes 9/8; local half offsets 697/868 in
+// shape 6, 471/564 in shape 9, and 551 on even steps without its streaming
+// stores; float32 (320 bytes: 803) 774/902 in shape 6, 816/891 in shape 7,
+// 778/983 in shape 9.  Even steps are bound by HBM.  Odd ones store rows
+// shifted by a node, which leave part of a sector at either end, and keep 18
+// addresses: the local storages take 168 registers there.  Staging the
+// stencil pays for the 16-bit storages, whose bytes are fewer than their
+// stencil's loads can hide behind; float32 is bound by its bytes either way.
 struct PipeCfg {
-  int by, minb_even, minb_odd, minb_even_local, minb_odd_local, zc, nb;
+  int by, minb_even, minb_odd, minb_even_local, minb_odd_local;
   bool ring;  // neighbour densities and adhesion sources also staged in
               // shared memory (a five-plane ring filled by the block)
   bool cs;    // streaming stores
 };
-// Measured on the 256^3 electrode: one plane in flight (nb = 2) beats two
-// (nb = 3, fewer blocks fit), and the best shapes are 8 rows for even steps
-// and 2 rows at 8 blocks per SM for odd steps.  Staging the neighbour
-// densities in a ring as well (shape 8) helps the half-offset odd step by
-// ~3 % and the local 16-bit even step by 6 %, and slows the float32 one (the
-// per-plane barrier); with streaming stores (shape 9) the local odd step
-// drops from 0.93 to 0.80 ms.
 __host__ __device__ constexpr PipeCfg pipe_cfg(int cfg) {
-  return cfg == 6   ? PipeCfg{8, 2, 2, 2, 2, 16, 2, false, false}
-         : cfg == 7 ? PipeCfg{2, 10, 8, 8, 6, 16, 2, false, false}
-         : cfg == 8 ? PipeCfg{2, 10, 8, 8, 6, 16, 2, true, false}
-         : cfg == 9 ? PipeCfg{2, 10, 8, 8, 6, 16, 2, true, true}
-                    : PipeCfg{4, 5, 4, 4, 3, 8, 2, false, false};
+  return cfg == 6   ? PipeCfg{8, 2, 2, 2, 2, false, false}
+         : cfg == 7 ? PipeCfg{2, 10, 8, 8, 6, false, false}
+         : cfg == 8 ? PipeCfg{2, 8, 8, 8, 6, true, false}
+         : cfg == 9 ? PipeCfg{2, 8, 8, 8, 6, true, true}
+                    : PipeCfg{4, 4, 4, 4, 3, true, true};
 }
-// Shared memory of a prefetching block: population buffers, then (ring)
-// five planes of (by + 2) x 34 density pairs and adhesion sources.
 constexpr int kPipeRingPlanes = 5, kPipeRingCols = kTile + 2;
-__host__ __device__ constexpr int pipe_smem_bytes(int cfg, int pair_bytes, bool pc) {
-  return pipe_cfg(cfg).nb * kQ * kTile * pipe_cfg(cfg).by * pair_bytes +
-         (pipe_cfg(cfg).ring ? kPipeRingPlanes * (pipe_cfg(cfg).by + 2) * kPipeRingCols *
-                                   (8 + 4 + (pc ? 4 : 0))
-                             : 0);
-}
 
 // Neighbour densities and adhesion sources from the shared-memory ring of a
 // prefetching block: row pointers of the node's ring row in planes z - 1,
@@ -573,22 +577,21 @@ __global__ void __launch_bounds__(DensityShape<CFG>::threads)
   const bool maybe_res = block_in_reservoir<S.by, S.bz>(p);
   if (x >= p.nx || y >= p.ny || z >= p.nz) return;
   const Geo g = make_geo(p, x, y, z);
-  float v1[kQ], v2[kQ];
-  load_pops<PARITY, ST>(p, w, g, v1, v2);
-  reservoir_state(p, maybe_res, x, y, z, v1, v2);
+  float2 v[kQ];
+  load_pops<PARITY, ST>(p, w, g, v);
+  reservoir_state(p, maybe_res, x, y, z, v);
   const int own = g.node(0, 0, 0);
-  if (in_bounds(w.fault, own, p.ntiles * kTile, kFaultRhoStore))
-    w.rho[own] = make_float2(sum19(v1), sum19(v2));
+  if (in_bounds(w.fault, own, p.ntiles * kTile, kFaultRhoStore)) w.rho[own] = sum19(v);
 }
 
 // ---- fused pass with prefetch ----
 // Shapes kCollidePipeFirst.. of the fused pass: each block owns 32 x by
-// nodes of a run of planes and walks the run plane by plane; every thread
-// copies the populations of its node in the next plane into shared memory
-// (cp.async, two buffers, the thread's own slots only, so no barrier) while
-// it collides the current plane.  The loads of one node overlap the
-// arithmetic of the one before without holding registers; the arithmetic is
-// that of k_collide_stream, so the results are bit-identical.
+// nodes of a run of planes and walks the run plane by plane, one warp per
+// row; a warp copies the populations of its row in the next plane into
+// shared memory (cp.async, two buffers of the warp's own, so no block
+// barrier) while it collides the current plane.  The loads of one plane
+// overlap the arithmetic of the one before without holding registers; the
+// arithmetic is that of k_collide_stream, so the results are bit-identical.
 template <typename T>
 __device__ __forceinline__ void cp_async(T *smem, const T *gmem) {
   static_assert(sizeof(T) == 4 || sizeof(T) == 8, "cp.async copies 4 or 8 bytes here");
@@ -596,6 +599,12 @@ __device__ __forceinline__ void cp_async(T *smem, const T *gmem) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(s), "l"(gmem),
                "n"((int)sizeof(T))
                : "memory");
+}
+// 16 bytes, both addresses 16-byte aligned, through L2 only: a population is
+// read once per launch, so it leaves L1 to the force stencil.
+__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() {
   asm volatile("cp.async.commit_group;\n" ::: "memory");
@@ -605,138 +614,298 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
+// Components of direction i for an i known only at run time (0, 1 or 2 for
+// -1, 0, 1), two bits each.
+__host__ __device__ constexpr unsigned long long packed_dir(int axis) {
+  unsigned long long v = 0;
+  for (int i = 0; i < kQ; ++i)
+    v |= (unsigned long long)((axis == 1 ? cy(i) : cz(i)) + 1) << (2 * i);
+  return v;
+}
+__device__ __forceinline__ int run_cy(int i) { return (int)((packed_dir(1) >> (2 * i)) & 3) - 1; }
+__device__ __forceinline__ int run_cz(int i) { return (int)((packed_dir(2) >> (2 * i)) & 3) - 1; }
+
+// The populations of one row of 32 nodes (x-tile bx, row y), plane by plane,
+// copied by one warp in 16-byte chunks.  Even steps read the tile itself,
+// one contiguous run.  Odd steps read population i from slot opp(i) of the
+// tile at (y - c_y, z - c_z), shifted by c_x: the slot's row of 32 is copied
+// whole, and the one node beyond its edge that a shifted read needs (lane 0
+// for c_x = 1, the last lane for c_x = -1) goes into element 32 of the row.
+// A chunk also carries values of nodes other rows own; they are not used, so
+// it does not matter that their owners may be replacing them.  Per warp and
+// plane this takes 5 (16-bit) or 10 (float32) copy instructions (odd steps:
+// one more and two integer operations each) instead of 19 with an address
+// each.
+template <int PARITY, typename T2>
+struct RowCopy {
+  static constexpr int kEl = 16 / (int)sizeof(T2);               // pairs per chunk
+  static constexpr int kStride = PARITY == 0 ? kTile : kTile + kEl;  // pairs per slot row
+  static constexpr int kPairs = kQ * kStride;                    // pairs per buffer
+  static constexpr int kChunks = kTilePairs / kEl;               // chunks per tile
+  static constexpr int kCopies = (kChunks + kTile - 1) / kTile;  // per lane
+  static constexpr int kOff = PARITY == 0 ? 1 : kCopies;
+  unsigned off[kOff];  // source (pairs) of this lane's chunks in the next plane
+  unsigned halo;       // source of this lane's edge node (lanes 0..9)
+  int at[3];           // element of a slot row this lane reads for c_x = -1, 0, 1
+  unsigned plane, total;
+
+  __device__ __forceinline__ RowCopy(const StepParams &p, int bx, int y, int z) {
+    const int lane = threadIdx.x;
+    plane = (unsigned)(p.ny * p.ntx) * (unsigned)kTilePairs;
+    total = plane * (unsigned)p.nz;
+    at[1] = lane;
+    if (PARITY == 0) {
+      off[0] = (unsigned)z * plane + (unsigned)(y * p.ntx + bx) * kTilePairs + lane * kEl;
+      return;
+    }
+    const int xlo = bx * kTile, xhi = min(xlo + kTile, p.nx) - 1;
+    at[0] = lane == xhi - xlo ? kTile : lane + 1;  // c_x = -1 reads x + 1
+    at[2] = lane == 0 ? kTile : lane - 1;
+#pragma unroll
+    for (int k = 0; k < kOff; ++k) {
+      const int c = lane + k * kTile;
+      const int i = min(c / (kTile / kEl), kQ - 1);
+      off[k] = source(p, i, bx, y, z) + (unsigned)(c % (kTile / kEl)) * kEl;
+    }
+    const int h = min(lane, 9);
+    const int i = h < 5 ? (h == 0 ? 1 : h + 3) : (h == 5 ? 10 : h + 7);
+    int x = h < 5 ? xhi + 1 : xlo - 1;
+    x = x < 0 ? p.nx - 1 : (x >= p.nx ? 0 : x);
+    halo = source(p, i, x / kTile, y, z) + (unsigned)(x % kTile);
+  }
+  // slot row of population i of row y, plane z, in x-tile xt (odd steps)
+  static __device__ __forceinline__ unsigned source(const StepParams &p, int i, int xt, int y,
+                                                    int z) {
+    int yw = y - run_cy(i), zw = z - run_cz(i);
+    yw = yw < 0 ? p.ny - 1 : (yw >= p.ny ? 0 : yw);
+    zw = zw < 0 ? p.nz - 1 : (zw >= p.nz ? 0 : zw);
+    const int slot = i == 0 ? 0 : (i <= 9 ? i + 9 : i - 9);
+    return (unsigned)((zw * p.ny + yw) * p.ntx + xt) * (unsigned)kTilePairs + slot * kTile;
+  }
+  // start copying the next plane of the run into buf and move on
+  __device__ __forceinline__ void next(const Workspace &w, T2 *buf) {
+    const T2 *f = static_cast<const T2 *>(w.f);
+    const int lane = threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < kCopies; ++k) {
+      const int c = lane + k * kTile;
+      if ((k + 1) * kTile > kChunks && c >= kChunks) break;
+      unsigned o = PARITY == 0 ? off[0] + k * kTile * kEl : off[k];
+      if (kChecked && !in_bounds(w.fault, (long long)o + kEl, (long long)total + 1, kFaultPopLoad))
+        o = 0;
+      T2 *dst = PARITY == 0 ? buf + c * kEl
+                            : buf + (c / (kTile / kEl)) * kStride + (c % (kTile / kEl)) * kEl;
+      cp_async16(dst, f + o);
+      if (PARITY == 1) off[k] = step(off[k]);
+    }
+    if (PARITY == 0) {
+      off[0] += plane;
+    } else {
+      if (lane < 10) {
+        const int i = lane < 5 ? (lane == 0 ? 1 : lane + 3) : (lane == 5 ? 10 : lane + 7);
+        unsigned o = halo;
+        if (kChecked && !in_bounds(w.fault, o, total, kFaultPopLoad)) o = 0;
+        cp_async(buf + i * kStride + kTile, f + o);
+      }
+      halo = step(halo);
+    }
+  }
+  // the same place one plane on, periodic
+  __device__ __forceinline__ unsigned step(unsigned o) const {
+    o += plane;
+    return min(o, o - total);
+  }
+  // population i of this lane's node
+  __device__ __forceinline__ T2 get(const T2 *buf, int i) const {
+    return buf[i * kStride + (PARITY == 0 ? at[1] : at[cx(i) + 1])];
+  }
+};
+
+// Where a block that walks along z finds a node's neighbours: the in-plane
+// part does not change from plane to plane.
+struct MarchGeo {
+  unsigned pin[3][3];  // pair offset of slot 0 of (x + dx, y + dy) inside a plane
+  unsigned pz[3];      // pair offset of planes z - 1, z, z + 1
+  unsigned plane, total;
+  __device__ __forceinline__ MarchGeo(const StepParams &p, int x, int y, int z) {
+    plane = (unsigned)(p.ny * p.ntx) * (unsigned)kTilePairs;
+    total = plane * (unsigned)p.nz;
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        int xw = x + a - 1, yw = y + b - 1;
+        xw = xw < 0 ? p.nx - 1 : (xw >= p.nx ? 0 : xw);
+        yw = yw < 0 ? p.ny - 1 : (yw >= p.ny ? 0 : yw);
+        pin[a][b] = (unsigned)(yw * p.ntx + xw / kTile) * (unsigned)kTilePairs + xw % kTile;
+      }
+    pz[1] = (unsigned)z * plane;
+    pz[0] = z == 0 ? total - plane : pz[1] - plane;
+    pz[2] = z == p.nz - 1 ? 0u : pz[1] + plane;
+  }
+  __device__ __forceinline__ void next() {
+    pz[0] = pz[1];
+    pz[1] = pz[2];
+    const unsigned o = pz[2] + plane;
+    pz[2] = min(o, o - total);
+  }
+  __device__ __forceinline__ unsigned pop_off(int dx, int dy, int dz) const {
+    return pz[dz + 1] + pin[dx + 1][dy + 1];
+  }
+};
+
+// Shared memory of a prefetching block: two buffers of its rows'
+// populations, n_s and (local storages) encoding densities, and with the
+// ring five planes of (by + 2) x 34 density pairs and adhesion sources.
+template <int PARITY, int ST, bool PC, int CFG>
+struct PipeSmem {
+  using T2 = typename Codec2<ST>::T2;
+  static constexpr PipeCfg P = pipe_cfg(CFG);
+  static constexpr int NT = kTile * P.by, kRing = (P.by + 2) * kPipeRingCols;
+  static constexpr bool L = storage_local(ST);
+  alignas(16) T2 pop[2][P.by][RowCopy<PARITY, T2>::kPairs];
+  float2 enc[L ? 2 : 1][L ? NT : 1];
+  float2 ring_rho[P.ring ? kPipeRingPlanes : 1][P.ring ? kRing : 1];
+  float ring_a[P.ring ? kPipeRingPlanes : 1][P.ring ? kRing : 1];
+  float ring_b[P.ring && PC ? kPipeRingPlanes : 1][P.ring && PC ? kRing : 1];
+  float ns[2][NT];
+  float ns2[PC ? 2 : 1][PC ? NT : 1];
+};
 
 // The fused pass of one block of a prefetching shape: x-tile bx, rows
 // [by0 * by, by0 * by + by) and the run of planes [bz * zc, bz * zc + zc)
 // of lattice (p, w).
 template <int PARITY, int ST, bool PC, int CFG>
-__device__ __forceinline__ void pipe_block(const StepParams &p, const Workspace &w, int bx,
+__device__ __forceinline__ void pipe_block(const StepParams &p, const Workspace &w, int zc, int bx,
                                            int by0, int bz) {
   using C = Codec2<ST>;
   using T2 = typename C::T2;
+  using Copy = RowCopy<PARITY, T2>;
   constexpr Shape S = CollideShape<PARITY, ST, CFG>::s;
   constexpr int NT = kTile * S.by;
-  constexpr PipeCfg P = pipe_cfg(CFG);
-  constexpr int ZC = P.zc, NB = P.nb, R = S.by + 2, RC = kPipeRingCols;
+  constexpr bool kRing = pipe_cfg(CFG).ring;
+  constexpr bool L = storage_local(ST);
+  constexpr int R = S.by + 2, RC = kPipeRingCols;
+  using Smem = PipeSmem<PARITY, ST, PC, CFG>;
   extern __shared__ __align__(16) unsigned char pipe_smem[];
-  T2(*buf)[kQ][NT] = reinterpret_cast<T2(*)[kQ][NT]>(pipe_smem);  // [NB][kQ][NT]
-  // ring: [5][R][RC] density pairs, then adhesion sources a_1 (and a_2)
-  float2 *ring_rho = reinterpret_cast<float2 *>(pipe_smem + NB * kQ * NT * sizeof(T2));
-  float *ring_a = reinterpret_cast<float *>(ring_rho + kPipeRingPlanes * R * RC);
-  float *ring_b = ring_a + kPipeRingPlanes * R * RC;
+  Smem &sm = *reinterpret_cast<Smem *>(pipe_smem);
   const int tid = threadIdx.y * kTile + threadIdx.x;
   const int x = bx * kTile + threadIdx.x, y = by0 * S.by + threadIdx.y;
-  const int z0 = bz * ZC, zend = min(z0 + ZC, p.nz);
+  const int z0 = bz * zc, zend = min(z0 + zc, p.nz);
   const int xlo = bx * kTile, ylo = by0 * S.by;
   const bool maybe_res = box_in_reservoir(p, xlo, min(xlo + kTile, p.nx) - 1, ylo,
                                           min(ylo + S.by, p.ny) - 1, z0, zend - 1);
-  const bool active = x < p.nx && y < p.ny;
-  // Without the ring no thread reads another's shared memory and idle
-  // threads may leave; with it every thread fills the ring and meets the
-  // per-plane barrier.
-  if (z0 >= zend || (!P.ring && !active)) return;
-  const T2 *f = static_cast<const T2 *>(w.f);
-  const long long pairs = p.ntiles * kTilePairs, nodes = p.ntiles * kTile;
-  auto prefetch = [&](int z, int b) {
-    if (!active) return;
-    const Geo g = make_geo(p, x, y, z);
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) {
-      const int slot = PARITY == 0 ? i : opp(i);
-      const T2 *src = f + (PARITY == 0 ? g.pop_off(0, 0, 0) : g.pop_off(-cx(i), -cy(i), -cz(i)));
-      if (kChecked && !in_bounds(w.fault, (src - f) + slot * kTile, pairs, kFaultPopLoad))
-        src = f - slot * kTile;
-      cp_async(&buf[b][i][tid], src + slot * kTile);
-    }
+  const bool row = y < p.ny;            // warp-uniform
+  const bool active = row && x < p.nx;
+  // Without the ring no warp reads another's shared memory and idle warps
+  // may leave; with it every thread fills the ring and meets the per-plane
+  // barrier.
+  if (z0 >= zend || (!kRing && !row)) return;
+  const long long nodes = p.ntiles * kTile;
+  const int plane_nodes = p.ny * p.ntx * kTile;
+  Copy copy(p, bx, row ? y : 0, z0);
+  // this node (padding lanes: their tile's lane, which exists)
+  int own = ((z0 * p.ny + (row ? y : 0)) * p.ntx + bx) * kTile + threadIdx.x;
+  auto prefetch = [&](int b, int n) {
+    if (!row) return;
+    copy.next(w, sm.pop[b][threadIdx.y]);
+    if (kChecked && !in_bounds(w.fault, n, nodes, kFaultGeometry)) n = 0;
+    cp_async(&sm.ns[b][tid], &w.ns[n]);
+    if (PC) cp_async(&sm.ns2[PC ? b : 0][PC ? tid : 0], &w.ns2[n]);
+    if (L) cp_async(&sm.enc[L ? b : 0][L ? tid : 0], &w.rho_enc[n]);
   };
   // ring plane of z (z0 - 1 <= z <= zend): rows y0 - 1 .. y0 + by, columns
-  // x0 - 1 .. x0 + 32, periodic
-  auto fill_ring = [&](int z) {
-    const int slot = (z - z0 + 1) % kPipeRingPlanes;
-    const int zw = z < 0 ? z + p.nz : (z >= p.nz ? z - p.nz : z);
-    for (int e = tid; e < R * RC; e += NT) {
-      const int r = e / RC, c = e % RC;
+  // x0 - 1 .. x0 + 32, periodic.  The in-plane nodes a thread copies are the
+  // same for every plane, so the wrapping is worked out once per block.
+  constexpr int RE = kRing ? (R * RC + NT - 1) / NT : 1;
+  int ring_node[RE];
+  if constexpr (kRing) {
+#pragma unroll
+    for (int k = 0; k < RE; ++k) {
+      const int e = tid + k * NT, r = e / RC, c = e % RC;
       int xw = xlo + c - 1, yw = ylo + r - 1;
       xw = xw < 0 ? xw + p.nx : (xw >= p.nx ? xw % p.nx : xw);
       yw = yw < 0 ? yw + p.ny : (yw >= p.ny ? yw % p.ny : yw);
-      long long n = ((long long)(zw * p.ny + yw) * p.ntx + xw / kTile) * kTile + xw % kTile;
+      ring_node[k] = (yw * p.ntx + xw / kTile) * kTile + xw % kTile;
+    }
+  }
+  auto fill_ring = [&](int z, int slot) {
+    const int zw = z < 0 ? z + p.nz : (z >= p.nz ? z - p.nz : z);
+    const long long plane = (long long)zw * plane_nodes;
+#pragma unroll
+    for (int k = 0; k < RE; ++k) {
+      const int e = tid + k * NT;
+      if (e >= R * RC) break;
+      long long n = plane + ring_node[k];
       if (kChecked && !in_bounds(w.fault, n, nodes, kFaultRhoLoad)) n = 0;
-      const int k = (slot * R + r) * RC + c;
-      cp_async(&ring_rho[k], &w.rho[n]);
-      cp_async(&ring_a[k], &w.ads[n]);
-      if (PC) cp_async(&ring_b[k], &w.ads2[n]);
+      if constexpr (kRing) {
+        cp_async(&sm.ring_rho[slot][e], &w.rho[n]);
+        cp_async(&sm.ring_a[slot][e], &w.ads[n]);
+        if (PC) cp_async(&sm.ring_b[PC ? slot : 0][PC ? e : 0], &w.ads2[n]);
+      }
     }
   };
-  if constexpr (!P.ring) {
-    // NB - 1 planes in flight; one commit group per plane (empty past the end)
-#pragma unroll
-    for (int d = 0; d + 1 < NB; ++d) {
-      if (z0 + d < zend) prefetch(z0 + d, d);
-      cp_async_commit();
-    }
-  } else {
-    prefetch(z0, 0);
-    fill_ring(z0 - 1);
-    fill_ring(z0);
-    fill_ring(z0 + 1);
-    cp_async_commit();
+  prefetch(0, own);
+  if constexpr (kRing) {
+    fill_ring(z0 - 1, 0);
+    fill_ring(z0, 1);
+    fill_ring(z0 + 1, 2);
   }
+  cp_async_commit();
+  MarchGeo mg(p, min(x, p.nx - 1), min(y, p.ny - 1), z0);
+  int slot = 0;  // ring slot of plane z - 1
   for (int z = z0; z < zend; ++z) {
-    const int b = (z - z0) % NB;
-    if constexpr (!P.ring) {
-      const int zp = z + NB - 1;
-      // buffer (zp - z0) % NB was consumed by the previous plane
-      if (zp < zend) prefetch(zp, (zp - z0) % NB);
-      cp_async_commit();
-      cp_async_wait<NB - 1>();  // the group of plane z is complete
-    } else {
-      // next plane's populations and the ring plane after it; the ring slot
-      // refilled here was last read two planes ago, before the previous
-      // barrier
-      if (z + 1 < zend) prefetch(z + 1, (z + 1 - z0) % NB);
-      if (z + 2 <= zend) fill_ring(z + 2);
-      cp_async_commit();
-      cp_async_wait<1>();   // this thread's copies for plane z are complete
-      __syncthreads();      // and every thread's ring copies too
-    }
-    if (!active) continue;
-    const Geo g = make_geo(p, x, y, z);
-    const int own = g.node(0, 0, 0);
-    const float2 own_prev =
-        storage_local(ST)
-            ? __ldg(&w.rho_enc[(kChecked && !in_bounds(w.fault, own, nodes, kFaultRhoLoad)) ? 0 : own])
-            : make_float2(0.f, 0.f);
-    float f1[kQ], f2[kQ];
+    const int b = (z - z0) & 1;
+    // next plane's populations and the ring plane after it; the ring slot
+    // refilled here was last read two planes ago, before the previous
+    // barrier, and the buffer in the previous plane, by this warp alone
+    __syncwarp();
+    if (z + 1 < zend) prefetch(b ^ 1, own + plane_nodes);
+    if (kRing && z + 2 <= zend)
+      fill_ring(z + 2, slot + 3 < kPipeRingPlanes ? slot + 3 : slot - 2);
+    cp_async_commit();
+    cp_async_wait<1>();  // this thread's copies for plane z are complete
+    if constexpr (kRing)
+      __syncthreads();   // and every thread's
+    else
+      __syncwarp();      // and every lane's
+    if (active) {
+      const T2 *buf = sm.pop[b][threadIdx.y];
+      const float2 own_prev = L ? sm.enc[L ? b : 0][L ? tid : 0] : make_float2(0.f, 0.f);
+      const float ns1 = sm.ns[b][tid];
+      const float2 ns = make_float2(ns1, PC ? sm.ns2[PC ? b : 0][PC ? tid : 0] : ns1);
+      float2 v[kQ];
 #pragma unroll
-    for (int i = 0; i < kQ; ++i) {
-      const float2 v = C::dec(buf[b][i][tid], dec_ref<ST>(p, own_prev, i));
-      f1[i] = v.x;
-      f2[i] = v.y;
-    }
-    reservoir_state(p, maybe_res, x, y, z, f1, f2);
-    if constexpr (!P.ring) {
-      collide_loaded<PARITY, ST, PC, GlobalRho, S.cs>(p, w, g, global_rho(p, w, g), f1, f2);
-    } else {
-      SmemStencil st;
-      const int r = threadIdx.y + 1;
+      for (int i = 0; i < kQ; ++i) v[i] = C::dec(copy.get(buf, i), dec_ref<ST>(p, own_prev, i));
+      reservoir_state(p, maybe_res, x, y, z, v);
+      if constexpr (!kRing) {
+        const Geo g = make_geo(p, x, y, z);
+        collide_loaded<PARITY, ST, PC, GlobalRho, S.cs>(p, w, mg, global_rho(p, w, g), v, ns);
+      } else {
+        SmemStencil st;
+        const int r = threadIdx.y + 1;
 #pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const int k = (((z - 1 + d) - z0 + 1) % kPipeRingPlanes * R + r) * RC;
-        st.rho[d] = ring_rho + k;
-        st.a[d] = ring_a + k;
-        st.b[d] = ring_b + k;
+        for (int d = 0; d < 3; ++d) {
+          const int sd = slot + d < kPipeRingPlanes ? slot + d : slot + d - kPipeRingPlanes;
+          st.rho[d] = sm.ring_rho[sd] + r * RC;
+          st.a[d] = sm.ring_a[sd] + r * RC;
+          st.b[d] = PC ? sm.ring_b[PC ? sd : 0] + (PC ? r * RC : 0) : nullptr;
+        }
+        st.c = threadIdx.x + 1;
+        collide_loaded<PARITY, ST, PC, SmemStencil, S.cs>(p, w, mg, st, v, ns);
       }
-      st.c = threadIdx.x + 1;
-      collide_loaded<PARITY, ST, PC, SmemStencil, S.cs>(p, w, g, st, f1, f2);
     }
+    slot = slot + 1 < kPipeRingPlanes ? slot + 1 : 0;
+    own += plane_nodes;
+    mg.next();
   }
 }
 
 template <int PARITY, int ST, bool PC, int CFG>
 __global__ void __launch_bounds__(CollideShape<PARITY, ST, CFG>::threads,
                                   CollideShape<PARITY, ST, CFG>::s.minb)
-    k_collide_pipe(StepParams p, Workspace w) {
-  pipe_block<PARITY, ST, PC, CFG>(p, w, blockIdx.x, blockIdx.y, blockIdx.z);
+    k_collide_pipe(StepParams p, Workspace w, int zc) {
+  pipe_block<PARITY, ST, PC, CFG>(p, w, zc, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
 template <int PARITY, int ST, int CFG, bool PC>
@@ -761,16 +930,15 @@ __global__ void __launch_bounds__(kTile * kFieldsBY * kFieldsBZ)
   const bool maybe_res = block_in_reservoir<kFieldsBY, kFieldsBZ>(p);
   if (x >= p.nx || y >= p.ny || z >= p.nz) return;
   const Geo g = make_geo(p, x, y, z);
-  float f1[kQ], f2[kQ];
-  load_pops<PARITY, ST>(p, w, g, f1, f2);
-  reservoir_state(p, maybe_res, x, y, z, f1, f2);
-  const float r1 = sum19(f1), r2 = sum19(f2);
-  float j1[3], j2[3];
-  first_moment(f1, j1);
-  first_moment(f2, j2);
-  float g1[3], g2[3];
+  float2 v[kQ];
+  load_pops<PARITY, ST>(p, w, g, v);
+  reservoir_state(p, maybe_res, x, y, z, v);
+  const float2 r = sum19(v);
+  const float r1 = r.x, r2 = r.y;
+  float2 j[3], gf[3];
+  first_moment(v, j);
   const float rho = r1 + r2;
-  force_per_mass<PC>(p, global_rho(p, w, g), w, g, rho, g1, g2);
+  force_per_mass<PC>(p, global_rho(p, w, g), rho, gf);
   int own = g.node(0, 0, 0);
   if (!in_bounds(w.fault, own, p.ntiles * kTile, kFaultGeometry)) own = 0;
   const float fluid = 1.0f - w.ns[own];
@@ -783,11 +951,11 @@ __global__ void __launch_bounds__(kTile * kFieldsBY * kFieldsBZ)
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     if (PC) {
-      const float m = fluid * (j1[d] + 0.5f * r1 * g1[d]) +
-                      fluid2 * (j2[d] + 0.5f * r2 * g2[d]);
+      const float m = fluid * (j[d].x + 0.5f * r1 * gf[d].x) +
+                      fluid2 * (j[d].y + 0.5f * r2 * gf[d].y);
       w.stage[(2 + d) * L + n] = m / rho;
     } else {
-      const float m = (j1[d] + 0.5f * r1 * g1[d]) + (j2[d] + 0.5f * r2 * g2[d]);
+      const float m = (j[d].x + 0.5f * r1 * gf[d].x) + (j[d].y + 0.5f * r2 * gf[d].y);
       w.stage[(2 + d) * L + n] = fluid * m / rho;
     }
   }
@@ -819,9 +987,9 @@ __global__ void k_init_equilibrium(StepParams p, Workspace w,
     if (storage_local(ST)) w.rho_enc[tn] = make_float2(r1, r2);
 #pragma unroll
     for (int i = 0; i < kQ; ++i) {
-      float2 ref = make_float2(p.ref[0][wclass(i)], p.ref[1][wclass(i)]);
-      if (storage_local(ST)) ref = make_float2(__fmul_rn(wgt(i), r1), __fmul_rn(wgt(i), r2));
-      b[i * kTile] = C::enc(__fmul_rn(wgt(i), r1), __fmul_rn(wgt(i), r2), ref);
+      const float2 f = make_float2(__fmul_rn(wgt(i), r1), __fmul_rn(wgt(i), r2));
+      // (local: the offset from the node's own density is zero)
+      b[i * kTile] = C::enc(f, storage_local(ST) ? mul2(f, pair_of(-C::kScale)) : p.nref[wclass(i)]);
     }
   }
 }
@@ -944,17 +1112,13 @@ __device__ __forceinline__ void wave_tile_item(const StepParams &p, const Worksp
       cp_async(&buf[b][i][tid], src + slot * kTile);
     }
   };
-  auto decode = [&](int b, int own, float (&v1)[kQ], float (&v2)[kQ]) {
+  auto decode = [&](int b, int own, float2 (&v)[kQ]) {
     const float2 own_prev =
         storage_local(ST)
             ? __ldg(&w.rho_enc[(kChecked && !in_bounds(w.fault, own, nodes, kFaultRhoLoad)) ? 0 : own])
             : make_float2(0.f, 0.f);
 #pragma unroll
-    for (int i = 0; i < kQ; ++i) {
-      const float2 v = C::dec(buf[b][i][tid], dec_ref<ST>(p, own_prev, i));
-      v1[i] = v.x;
-      v2[i] = v.y;
-    }
+    for (int i = 0; i < kQ; ++i) v[i] = C::dec(buf[b][i][tid], dec_ref<ST>(p, own_prev, i));
   };
   const int grp = (int)(k / (unsigned)a.tp), T = (int)(k % (unsigned)a.tp);
   const int tx = T % p.ntx, ty = T / p.ntx;
@@ -993,19 +1157,19 @@ __device__ __forceinline__ void wave_tile_item(const StepParams &p, const Worksp
   if (has_c && active) {
     cp_async_wait<1>();
     const Geo g = make_geo(p, x, y, q);
-    float f1[kQ], f2[kQ];
-    decode(0, g.node(0, 0, 0), f1, f2);
-    reservoir_state(p, box_in_reservoir(p, xlo, xhi, ylo, yhi, q, q), x, y, q, f1, f2);
-    collide_loaded<PARITY, ST, PC, WaveRho>(p, w, g, WaveRho{global_rho(p, w, g)}, f1, f2);
+    float2 v[kQ];
+    decode(0, g.node(0, 0, 0), v);
+    reservoir_state(p, box_in_reservoir(p, xlo, xhi, ylo, yhi, q, q), x, y, q, v);
+    collide_loaded<PARITY, ST, PC, WaveRho>(p, w, g, WaveRho{global_rho(p, w, g)}, v,
+                                            node_ns<PC>(p, w, g));
   }
   cp_async_wait<0>();
   if (has_d && active) {
     const long long own = ((long long)(zd * p.ny + y) * p.ntx + tx) * kTile + threadIdx.x;
-    float v1[kQ], v2[kQ];
-    decode(1, (int)own, v1, v2);
-    reservoir_state(p, box_in_reservoir(p, xlo, xhi, ylo, yhi, zd, zd), x, y, zd, v1, v2);
-    if (in_bounds(w.fault, own, nodes, kFaultRhoStore))
-      w.rho[own] = make_float2(sum19(v1), sum19(v2));
+    float2 v[kQ];
+    decode(1, (int)own, v);
+    reservoir_state(p, box_in_reservoir(p, xlo, xhi, ylo, yhi, zd, zd), x, y, zd, v);
+    if (in_bounds(w.fault, own, nodes, kFaultRhoStore)) w.rho[own] = sum19(v);
   }
   __syncthreads();  // the tile's densities are stored, the buffers free
   if (has_d && tid == 0) {
@@ -1128,10 +1292,10 @@ struct RingRho {
 template <int PARITY, int ST>
 __device__ __forceinline__ float2 node_density(const StepParams &p, const Workspace &w,
                                                const Geo &g, int x, int y, int z) {
-  float v1[kQ], v2[kQ];
-  load_pops<PARITY, ST>(p, w, g, v1, v2);
-  reservoir_state(p, p.res.any != 0, x, y, z, v1, v2);
-  return make_float2(sum19(v1), sum19(v2));
+  float2 v[kQ];
+  load_pops<PARITY, ST>(p, w, g, v);
+  reservoir_state(p, p.res.any != 0, x, y, z, v);
+  return sum19(v);
 }
 
 template <int PARITY, int ST, bool PC>
@@ -1260,15 +1424,14 @@ __global__ void __launch_bounds__(kTile * kBatchBY)
   if (!batch_coords(a, r, x, y, z, maybe_res)) return;
   const BatchItem &it = a.item[r];
   const Geo g = make_geo(it.p, x, y, z);
-  float v1[kQ], v2[kQ];
+  float2 v[kQ];
   if (it.parity == 0)
-    load_pops<0, ST>(it.p, it.w, g, v1, v2);
+    load_pops<0, ST>(it.p, it.w, g, v);
   else
-    load_pops<1, ST>(it.p, it.w, g, v1, v2);
-  reservoir_state(it.p, maybe_res, x, y, z, v1, v2);
+    load_pops<1, ST>(it.p, it.w, g, v);
+  reservoir_state(it.p, maybe_res, x, y, z, v);
   const int own = g.node(0, 0, 0);
-  if (in_bounds(it.w.fault, own, it.p.ntiles * kTile, kFaultRhoStore))
-    it.w.rho[own] = make_float2(sum19(v1), sum19(v2));
+  if (in_bounds(it.w.fault, own, it.p.ntiles * kTile, kFaultRhoStore)) it.w.rho[own] = sum19(v);
 }
 
 // All items of one launch have per-component fractions (PC) or none do.
@@ -1287,9 +1450,8 @@ __global__ void __launch_bounds__(kTile * kBatchBY, CollideShape<1, ST, 0>::s.mi
 
 // Blocks per SM the batched prefetching pass is compiled for: those of the
 // single-lattice kernel, except the local storages' odd step in shape 9,
-// whose budget (6 blocks, up to 170 registers) lets the lattice lookup take
-// it to 137 registers and 7 resident blocks; held to 8 blocks (128
-// registers) it needs no spill.
+// which runs faster held to 8 blocks (128 registers, no spill) than at 6:
+// 567 against 576 us a step over twelve lattices of 36^3 .. 160^3.
 template <int PARITY, int ST, int CFG>
 __host__ __device__ constexpr int batch_pipe_minb() {
   return (storage_local(ST) && PARITY == 1 && CFG == 9) ? 8
@@ -1299,7 +1461,7 @@ __host__ __device__ constexpr int batch_pipe_minb() {
 // The prefetching fused pass over a batch of lattices at one AA parity:
 // item r's blocks (prefix[r] .. prefix[r + 1]) tile its lattice as
 // k_collide_pipe's grid does for shape CFG (gx x-tiles, gy row groups, runs
-// of zc planes), and each block runs that kernel's body on its lattice.
+// of its zc planes), and each block runs that kernel's body on its lattice.
 template <int PARITY, int ST, bool PC, int CFG>
 __global__ void __launch_bounds__(CollideShape<PARITY, ST, CFG>::threads,
                                   batch_pipe_minb<PARITY, ST, CFG>())
@@ -1308,7 +1470,7 @@ __global__ void __launch_bounds__(CollideShape<PARITY, ST, CFG>::threads,
   const BatchItem &it = a.item[r];
   const int lb = blockIdx.x - a.prefix[r];
   const int rest = lb / it.gx;
-  pipe_block<PARITY, ST, PC, CFG>(it.p, it.w, lb % it.gx, rest % it.gy, rest / it.gy);
+  pipe_block<PARITY, ST, PC, CFG>(it.p, it.w, it.zc, lb % it.gx, rest % it.gy, rest / it.gy);
 }
 
 }  // namespace

@@ -49,53 +49,93 @@ __host__ __device__ constexpr int wclass(int i) {
 // Half offsets are kept scaled by 2^14 (see above).
 constexpr float kHalfScale = 16384.0f, kHalfUnscale = 1.0f / 16384.0f;
 
-// The stored pair (sigma = 1, 2) of one direction at one node.  enc_s
-// takes the reference already multiplied by kScale (exact: a power of two),
-// so the half encode is one fused multiply-add per value: f * 2^14 - r 2^14
-// rounds to the same float as (f - r) * 2^14 because scaling by a power of
-// two commutes with rounding.
+// Packed arithmetic on the pair (sigma = 1, 2): one instruction does both
+// components, each rounded as the scalar operation would be (add.f32x2,
+// mul.f32x2, fma.f32x2).  Both components take the same steps everywhere on
+// the path, and the 16-bit fused passes are bound by instruction issue
+// (1,115-1,289 instructions a node in scalar form), so the pairs stay pairs
+// from the load to the store.  A subtraction is a fused multiply-add with
+// -1, which rounds once like the subtraction it stands for.
+// A packed product that feeds a packed sum is fused with it by the assembler
+// (measured: mul2 into add2 rounds once, .rn or not), so where both roundings
+// matter one of the two operations is written scalar.
+#ifdef __CUDACC__
+__device__ __forceinline__ unsigned long long pack2(float2 v) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(v.x), "f"(v.y));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ float2 pair_of(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+  return unpack2(r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+  return unpack2(r);
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)), "l"(pack2(c)));
+  return unpack2(r);
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, pair_of(-1.0f), a); }
+#endif
+
+// The stored pair (sigma = 1, 2) of one direction at one node.  enc takes
+// the negated reference already multiplied by kScale (exact: a power of
+// two), so the half encode is one fused multiply-add per value: f * 2^14 -
+// r 2^14 rounds to the same float as (f - r) * 2^14 because scaling by a
+// power of two commutes with rounding.
 template <int ST> struct Codec2;
 template <> struct Codec2<kF32> {
   using T2 = float2;
   static constexpr float kScale = 1.0f;
   static __device__ __forceinline__ float2 dec(T2 v, float2) { return v; }
-  static __device__ __forceinline__ T2 enc_s(float f1, float f2, float2) {
-    return make_float2(f1, f2);
-  }
-  static __device__ __forceinline__ T2 enc(float f1, float f2, float2) {
-    return make_float2(f1, f2);
-  }
+  static __device__ __forceinline__ T2 enc(float2 f, float2) { return f; }
 };
 template <> struct Codec2<kF16> {
   using T2 = __half2;
   static constexpr float kScale = kHalfScale;
   static __device__ __forceinline__ float2 dec(T2 v, float2 r) {
-    const float2 h = __half22float2(v);
-    return make_float2(fmaf(h.x, kHalfUnscale, r.x), fmaf(h.y, kHalfUnscale, r.y));
+    return fma2(__half22float2(v), pair_of(kHalfUnscale), r);
   }
-  static __device__ __forceinline__ T2 enc_s(float f1, float f2, float2 rs) {
-    return __floats2half2_rn(fmaf(f1, kHalfScale, -rs.x), fmaf(f2, kHalfScale, -rs.y));
-  }
-  static __device__ __forceinline__ T2 enc(float f1, float f2, float2 r) {
-    return enc_s(f1, f2, make_float2(r.x * kHalfScale, r.y * kHalfScale));
+  static __device__ __forceinline__ T2 enc(float2 f, float2 nrs) {
+    const float2 o = fma2(f, pair_of(kHalfScale), nrs);
+    return __floats2half2_rn(o.x, o.y);
   }
 };
 template <> struct Codec2<kBF16> {
   using T2 = __nv_bfloat162;
   static constexpr float kScale = 1.0f;
   static __device__ __forceinline__ float2 dec(T2 v, float2 r) {
-    const float2 h = __bfloat1622float2(v);
-    return make_float2(r.x + h.x, r.y + h.y);
+    return add2(r, __bfloat1622float2(v));
   }
-  static __device__ __forceinline__ T2 enc_s(float f1, float f2, float2 r) {
-    return __floats2bfloat162_rn(f1 - r.x, f2 - r.y);
-  }
-  static __device__ __forceinline__ T2 enc(float f1, float f2, float2 r) {
-    return enc_s(f1, f2, r);
+  static __device__ __forceinline__ T2 enc(float2 f, float2 nr) {
+    const float2 o = add2(f, nr);
+    return __floats2bfloat162_rn(o.x, o.y);
   }
 };
-template <> struct Codec2<kF16L> : Codec2<kF16> {};
-template <> struct Codec2<kBF16L> : Codec2<kBF16> {};
+// enc_local: the reference is w rho, rho the destination's density.  The
+// bfloat16 offset rounds w rho first, as the decode does: scalar products,
+// see the packed operations above.
+template <> struct Codec2<kF16L> : Codec2<kF16> {
+  static __device__ __forceinline__ T2 enc_local(float2 f, float w, float2 rho) {
+    return enc(f, mul2(pair_of(-(w * kScale)), rho));
+  }
+};
+template <> struct Codec2<kBF16L> : Codec2<kBF16> {
+  static __device__ __forceinline__ T2 enc_local(float2 f, float w, float2 rho) {
+    return enc(f, make_float2(__fmul_rn(-w, rho.x), __fmul_rn(-w, rho.y)));
+  }
+};
 
 // D3Q19 velocity set in the order of Eq. A.8: direction i + 9 is the
 // opposite of direction i (i = 1..9).
@@ -175,7 +215,8 @@ struct StepParams {
   float tau[2];
   float G;
   float F[3];
-  float ref[2][3];   // *_OFFSET storages: w_class * rho0_sigma (float product)
+  float2 ref[3];     // *_OFFSET storages: w_class * rho0_sigma (float product)
+  float2 nref[3];    // the same negated and times the codec's scale (encoding)
   int storage;       // StorageKind
   Reservoirs res;
 };
@@ -242,7 +283,8 @@ __host__ __device__ inline long long wave_flag_words(long long nx, long long ny,
   return nz * ny * ((nx + 31) / 32);
 }
 
-constexpr int kRedBlocks = 304;  // 2 x 152 SMs
+constexpr int kSms = 152;        // SMs of a GB300
+constexpr int kRedBlocks = 2 * kSms;
 constexpr int kRedThreads = 256;
 constexpr int kRedK = 11;        // mass[2], sat num/den, p_face[6], nonfinite
 
@@ -274,6 +316,7 @@ struct BatchItem {
   Workspace w;
   int parity;  // AA parity of this lattice's current time step
   int gx, gy;  // blocks along x and y
+  int zc;      // planes per block (prefetching fused pass)
 };
 struct BatchArgs {
   int n;

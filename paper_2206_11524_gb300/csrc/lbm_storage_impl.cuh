@@ -36,12 +36,28 @@ void density_any(const StepParams &p, const Workspace &w, int cfg, cudaStream_t 
     default: density_cfg<PARITY, 0>(p, w, s);
   }
 }
+// Planes per block of the prefetching fused pass over n lattices that take
+// columns[k] blocks of 32 x by nodes side by side and nz[k] planes.  A block
+// pays for its set-up and its first, exposed copies once per run, so runs
+// are as long as they can be, up to 16 planes, while the blocks still make
+// one and a half rounds of 16 warps on every SM: with fewer, SMs stand idle.
+// Measured (us, even / odd step; runs of 16, 8, 4, 2, 1 planes): 32 x 16 x 16
+// float32 31/27, 18/16, 12/12, 9/9, 9/9; 48^3 local half offsets 23/23,
+// 15/14, 12/13, 12/14, 12/14; 128^3 72/83, 72/82, 72/82, 76/92, 92/119;
+// 256^3 float32 774/890 (16) against 760/926 (4).
+int pipe_run(const long long *columns, const int *nz, int n, int by) {
+  const long long want = (long long)kSms * 24 / by;
+  for (int zc = 16; zc > 1; zc /= 2) {
+    long long blocks = 0;
+    for (int k = 0; k < n; ++k) blocks += columns[k] * ((nz[k] + zc - 1) / zc);
+    if (blocks >= want) return zc;
+  }
+  return 1;
+}
 template <int PARITY, bool PC, int CFG>
 void collide_pipe_launch(const StepParams &p, const Workspace &w, cudaStream_t s) {
-  using T2 = typename Codec2<kST>::T2;
   constexpr Shape S = CollideShape<PARITY, kST, CFG>::s;
-  constexpr PipeCfg P = pipe_cfg(CFG);
-  constexpr int smem = pipe_smem_bytes(CFG, (int)sizeof(T2), PC);
+  constexpr int smem = (int)sizeof(PipeSmem<PARITY, kST, PC, CFG>);
   // the shared-memory limit is an attribute of the function on each device;
   // if setting it fails, the launch below reports the error
   static std::once_flag attr_once[16];
@@ -51,8 +67,11 @@ void collide_pipe_launch(const StepParams &p, const Workspace &w, cudaStream_t s
       cudaFuncSetAttribute(k_collide_pipe<PARITY, kST, PC, CFG>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     });
-  const dim3 grid(p.ntx, (p.ny + S.by - 1) / S.by, (p.nz + P.zc - 1) / P.zc);
-  k_collide_pipe<PARITY, kST, PC, CFG><<<grid, dim3(kTile, S.by, 1), smem, s>>>(p, w);
+  const int gy = (p.ny + S.by - 1) / S.by;
+  const long long columns = (long long)p.ntx * gy;
+  const int zc = pipe_run(&columns, &p.nz, 1, S.by);
+  const dim3 grid(p.ntx, gy, (p.nz + zc - 1) / zc);
+  k_collide_pipe<PARITY, kST, PC, CFG><<<grid, dim3(kTile, S.by, 1), smem, s>>>(p, w, zc);
 }
 template <int PARITY, int CFG>
 void collide_pipe_cfg(const StepParams &p, const Workspace &w, cudaStream_t s) {
@@ -368,26 +387,31 @@ namespace {
 // k_batch_collide_pipe over the items of `a` at AA parity PARITY, shape CFG.
 template <int PARITY, bool PC, int CFG>
 cudaError_t batch_pipe_launch(const BatchArgs &a, cudaStream_t s) {
-  using T2 = typename Codec2<kST>::T2;
   constexpr Shape S = CollideShape<PARITY, kST, CFG>::s;
-  constexpr PipeCfg P = pipe_cfg(CFG);
-  constexpr int smem = pipe_smem_bytes(CFG, (int)sizeof(T2), PC);
+  constexpr int smem = (int)sizeof(PipeSmem<PARITY, kST, PC, CFG>);
   static thread_local BatchArgs b;  // ~16 KB: kept off the stack
   b.n = 0;
-  b.prefix[0] = 0;
+  long long columns[kBatchMax];
+  int nz[kBatchMax];
   for (int k = 0; k < a.n; ++k) {
     if ((a.item[k].parity & 1) != PARITY) continue;
     BatchItem &it = b.item[b.n];
     it = a.item[k];
     it.gx = it.p.ntx;
     it.gy = (it.p.ny + S.by - 1) / S.by;
-    const long long blocks =
-        (long long)b.prefix[b.n] + (long long)it.gx * it.gy * ((it.p.nz + P.zc - 1) / P.zc);
-    if (blocks > 2147483647LL) return cudaErrorInvalidValue;
-    b.prefix[b.n + 1] = (int)blocks;
+    columns[b.n] = (long long)it.gx * it.gy;
+    nz[b.n] = it.p.nz;
     ++b.n;
   }
   if (b.n == 0) return cudaSuccess;
+  const int zc = pipe_run(columns, nz, b.n, S.by);  // one length: the lattices share the SMs
+  b.prefix[0] = 0;
+  for (int k = 0; k < b.n; ++k) {
+    b.item[k].zc = zc;
+    const long long blocks = (long long)b.prefix[k] + columns[k] * ((nz[k] + zc - 1) / zc);
+    if (blocks > 2147483647LL) return cudaErrorInvalidValue;
+    b.prefix[k + 1] = (int)blocks;
+  }
   // the shared-memory limit is an attribute of the function on each device
   static std::once_flag attr_once[16];
   static cudaError_t attr_err[16];

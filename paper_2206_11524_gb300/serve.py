@@ -122,12 +122,6 @@ def make_requests(n_req=32, seed=2206, L_min=32, L_max=192, steps_min=1000,
 # slower than the two batched passes.
 WAVE_BATCH = 0
 
-# Fused-pass shapes (density, even, odd) of the served lattices where they
-# differ from the library's defaults, which were tuned on one 256^3 lattice:
-# half-offset lattices of this trace step faster batched in 32 x 2 tiles
-# (16,345 against 15,707 MLUPS over 24 requests of the trace).
-SERVE_LAUNCH = {"f16": (0, 7, 7)}
-
 
 def _lattice_for(req: Request, storage: str, stream, wave=WAVE_BATCH):
     lat = lbm.Lattice(req.L, req.L, req.L, tau=req.tau, G=req.G, stream=stream,
@@ -136,8 +130,6 @@ def _lattice_for(req: Request, storage: str, stream, wave=WAVE_BATCH):
     for face, (Lr, a, b) in req.reservoirs.items():
         lat.set_bc(face, Lr, a, b)
     lat.init_equilibrium(req.rho_a, req.rho_b)
-    if storage in SERVE_LAUNCH:
-        lat.set_launch_config(*SERVE_LAUNCH[storage])
     lat.set_wavefront(wave)
     return lat
 
