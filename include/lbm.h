@@ -170,10 +170,14 @@ LBM_API lbm_status lbm_set_bc_velocity(lbm_ctx *ctx, int face, int layers,
  * the context's stream.  Each step launches the density pass and the fused
  * force/collide/bounce-back/stream pass, or the single-pass sweep when
  * lbm_set_single_pass enabled it, or the wavefront launch when
- * lbm_set_wavefront enabled it.  n_steps = 0 is a no-op.  EINTERNAL (and
+ * lbm_set_wavefront enabled it.  A small lattice (up to 4,608 x-tiles: nx /
+ * 32, rounded up, times ny nz) without those two settings and without launch
+ * shapes of the caller's (lbm_set_launch_config) takes up to 256 steps per
+ * launch instead, with the same results bit for bit; its waits are bounded
+ * like the wavefront's.  n_steps = 0 is a no-op.  EINTERNAL (and
  * nothing enqueued) when a device fault was reported for the current state:
- * by a synchronising call (below), or by a wavefront launch that already
- * ran, through a host-mapped word the kernel sets (no stream wait). */
+ * by a synchronising call (below), or by a launch that already ran, through
+ * a host-mapped word the kernel sets (no stream wait). */
 LBM_API lbm_status lbm_step(lbm_ctx *ctx, int n_steps);
 
 /* Single-pass stepping for lbm_step (planes > 0; 0 = two passes, the
@@ -214,8 +218,10 @@ LBM_API lbm_status lbm_set_wavefront(lbm_ctx *ctx, int shape, int lag);
  * x / 32, T = ceil(ny / by) * ceil(nx / 32), of one tile's density flag that
  * the launch then never publishes, so the collisions that read those
  * densities wait until their limit runs out (-1 = none, the default).  In a
- * batch they apply when this context is the first one.  EINVAL if the index
- * is outside the flag words. */
+ * batch they apply when this context is the first one.  In the launches of
+ * small lattices beyond 128 x-tiles (lbm_step) spin_limit bounds each
+ * barrier's polls, and any withheld flag keeps the first barrier from
+ * completing.  EINVAL if the index is outside the flag words. */
 LBM_API lbm_status lbm_set_wavefront_limits(lbm_ctx *ctx, uint32_t spin_limit,
                                             int64_t withhold_flag);
 /* The wavefront shape (0: off) and lag in use, to *shape and *lag (either
@@ -277,8 +283,9 @@ LBM_API const char *lbm_last_error(const lbm_ctx *ctx);
  * stores).  A new context starts with the shapes measured fastest for its
  * storage on a 256^3 lattice (float32 1/6/7, half and bfloat16 offsets 0/9/8,
  * local offsets 0/9/9).  Results do not depend on the choice; speed does (the
- * autotuner measures them per lattice size and storage).  EINVAL if out of
- * range. */
+ * autotuner measures them per lattice size and storage).  Once they are set,
+ * lbm_step runs the two passes in them, small lattices included.  EINVAL if
+ * out of range. */
 #define LBM_DENSITY_CONFIGS 3
 #define LBM_COLLIDE_CONFIGS 10
 LBM_API lbm_status lbm_set_launch_config(lbm_ctx *ctx, int density_cfg,

@@ -126,10 +126,13 @@ def tune(nx, ny, nz, storage="f32", reps=10, single_pass=False, margin=0.03,
     against the wavefront step at WAVE_CANDIDATES (with `wavefront`) and, with
     single_pass, against the single-pass step at box depths that fit the SM
     count; another step than the two-pass one is kept only if it is faster by
-    more than `margin` (single-pass depth 0 and wavefront shape 0 otherwise)."""
+    more than `margin` (single-pass depth 0 and wavefront shape 0 otherwise).
+    Where the library's own choice for an untuned lattice (several steps per
+    launch on small ones) beats all of them by `margin`, the shapes are -1:
+    none are set."""
     lat = _scratch(nx, ny, nz, storage)
     ctx = lat.ctx
-    timings = {"density": [], "even": [], "odd": []}
+    timings = {"density": [], "even": [], "odd": [], "untuned_step": _step_ms(lat)}
     for d in range(lbm.LBM_DENSITY_CONFIGS):
         lbm.lbm_set_launch_config(ctx, d, 0, 0)
         timings["density"].append(_time(lat, lambda: lbm.lbm_density(ctx), reps))
@@ -187,6 +190,8 @@ def tune(nx, ny, nz, storage="f32", reps=10, single_pass=False, margin=0.03,
                 if ms < best_ms:
                     best_sp, best_wave, best_ms = planes, (0, 0), ms
             lat.set_single_pass(0)
+        if timings["untuned_step"] < best_ms * (1.0 - margin):
+            cfg, best_sp, best_wave = (-1, -1, -1), 0, (0, 0)
     lat.close()
     return cfg + (best_sp,) + best_wave, timings
 
@@ -206,7 +211,8 @@ def apply(lattice, table: TuneTable | None = None, tune_if_missing=True,
                             wavefront=wavefront)
         table.put(nx, ny, nz, storage, cfg, timings)
     if cfg is not None:
-        lbm.lbm_set_launch_config(lattice.ctx, *cfg[:3])
+        if cfg[0] >= 0:
+            lbm.lbm_set_launch_config(lattice.ctx, *cfg[:3])
         lattice.set_single_pass(cfg[3] if len(cfg) > 3 else 0)
         lattice.set_wavefront(*(cfg[4:6] if len(cfg) > 5 else (0, 0)))
     return cfg

@@ -41,6 +41,7 @@ struct lbm_ctx {
   bool have_state;
   uint64_t bc_version;    // bumped by every lbm_set_bc
   int launch_cfg[3];      // launch shapes: density, even fused, odd fused
+  bool launch_cfg_set;    // by the caller: lbm_step keeps the passes they are for
   int single_pass_zc;     // > 0: lbm_step sweeps once, boxes of this many planes
   int wave_cfg;           // > 0: lbm_step is one wavefront launch of this shape
   int wave_lag;           // planes between a plane's density and its collision
@@ -370,6 +371,7 @@ lbm_status lbm_create(const lbm_params *params, void *d_workspace,
   c->launch_cfg[0] = f32 ? 1 : 0;
   c->launch_cfg[1] = f32 ? 6 : 9;
   c->launch_cfg[2] = f32 ? 7 : local ? 9 : 8;
+  c->launch_cfg_set = false;
   c->single_pass_zc = 0;
   c->wave_cfg = 0;
   c->wave_lag = hmcsc::kWaveLagDefault;
@@ -668,6 +670,23 @@ lbm_status lbm_step(lbm_ctx *c, int n_steps) {
                 "load a checkpoint or set a new state");
   }
   for (int k = 0; k < n_steps; ++k) {
+    // small lattices stay on the device for several steps; a reservoir change
+    // takes effect at the end of a step, so the step it was made for is taken
+    // on its own
+    if (c->wave_cfg == 0 && c->single_pass_zc == 0 && !c->launch_cfg_set &&
+        c->sp.ntiles <= hmcsc::kResidentTiles &&
+        memcmp(&c->sp.res, &c->res_current, sizeof(hmcsc::Reservoirs)) == 0) {
+      const int m = n_steps - k < hmcsc::kResidentSteps ? n_steps - k : hmcsc::kResidentSteps;
+      cudaError_t e = hmcsc::launch_resident(c->sp, c->ws, parity(c), m, c->wave_spin,
+                                             c->wave_hold >= 0, c->stream);
+      if (e != cudaSuccess) return cuda_fail(c, e, "resident kernel");
+      for (int q = 0; q < m; ++q) {
+        c->rho_at = c->t;
+        finish_step(c);
+      }
+      k += m - 1;
+      continue;
+    }
     if (c->wave_cfg > 0) {
       cudaError_t e = hmcsc::launch_wave(c->sp, c->ws, parity(c), c->wave_cfg, c->wave_lag,
                                          c->wave_spin, c->wave_hold, c->stream);
@@ -1118,6 +1137,7 @@ lbm_status lbm_set_launch_config(lbm_ctx *c, int density_cfg, int even_cfg,
   c->launch_cfg[0] = density_cfg;
   c->launch_cfg[1] = even_cfg;
   c->launch_cfg[2] = odd_cfg;
+  c->launch_cfg_set = true;
   return LBM_OK;
 }
 

@@ -93,18 +93,20 @@ __device__ __forceinline__ float2 dec_ref(const StepParams &p, float2 own_prev,
 }
 
 // The 19 populations of both components at the current time step, decoded
-// to float32.
-template <int PARITY, int ST>
+// to float32.  MUT: the encoding densities may have been written earlier in
+// the same launch, so they are not read through the read-only path.
+template <int PARITY, int ST, bool MUT = false>
 __device__ __forceinline__ void load_pops(const StepParams &p, const Workspace &w,
                                           const Geo &g, float2 (&v)[kQ]) {
   using C = Codec2<ST>;
   const typename C::T2 *f = static_cast<const typename C::T2 *>(w.f);
   const long long nodes = p.ntiles * kTile, pairs = p.ntiles * kTilePairs;
-  const int own = g.node(0, 0, 0);
-  const float2 own_prev =
-      storage_local(ST)
-          ? __ldg(&w.rho_enc[(kChecked && !in_bounds(w.fault, own, nodes, kFaultRhoLoad)) ? 0 : own])
-          : make_float2(0.f, 0.f);
+  int own = g.node(0, 0, 0);
+  float2 own_prev = make_float2(0.f, 0.f);
+  if (storage_local(ST)) {
+    if (kChecked && !in_bounds(w.fault, own, nodes, kFaultRhoLoad)) own = 0;
+    own_prev = MUT ? __ldca(&w.rho_enc[own]) : __ldg(&w.rho_enc[own]);
+  }
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
     // population i of node x: slot i at x (even), slot opp(i) at x - c_i (odd)
@@ -177,6 +179,8 @@ struct GlobalRho {  // the density array written by the density pass
   __device__ __forceinline__ float a2(int dx, int dy, int dz) const {
     return __ldg(&ads2[gidx(dx, dy, dz)]);
   }
+  template <bool PC>
+  __device__ __forceinline__ void adhesion(float2 (&A)[3]) const;
 };
 __device__ __forceinline__ GlobalRho global_rho(const StepParams &p, const Workspace &w,
                                                 const Geo &g) {
@@ -195,41 +199,56 @@ __device__ __forceinline__ GlobalRho global_rho(const StepParams &p, const Works
 // fused into the sum it enters, written out so that each kernel rounds alike.
 // gf[d] = (g_1, g_2) along axis d.
 template <bool PC, typename RS>
-__device__ __forceinline__ void force_per_mass(const StepParams &p, const RS &rs,
-                                               float rho_tot, float2 (&gf)[3]) {
-  float2 s[3], sab[3];  // (S_1, S_2) and (A_1, A_2), the latter when PC
-  float sa[3];          // A otherwise
+__device__ __forceinline__ void adhesion_sum(const RS &rs, float2 (&A)[3]) {
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    s[d] = sab[d] = pair_of(0.0f);
-    sa[d] = 0.0f;
-  }
+  for (int d = 0; d < 3; ++d) A[d] = pair_of(0.0f);
 #pragma unroll
   for (int i = 1; i <= 9; ++i) {
-    const float2 dr = sub2(rs.at(cx(i), cy(i), cz(i)), rs.at(-cx(i), -cy(i), -cz(i)));
     const float da1 = __fsub_rn(rs.a1(cx(i), cy(i), cz(i)), rs.a1(-cx(i), -cy(i), -cz(i)));
-    float2 da = pair_of(0.0f);
-    if (PC) da = make_float2(da1, __fsub_rn(rs.a2(cx(i), cy(i), cz(i)),
-                                            rs.a2(-cx(i), -cy(i), -cz(i))));
+    float da2 = 0.0f;
+    if (PC) da2 = __fsub_rn(rs.a2(cx(i), cy(i), cz(i)), rs.a2(-cx(i), -cy(i), -cz(i)));
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const int c = d == 0 ? cx(i) : d == 1 ? cy(i) : cz(i);
       if (c == 0) continue;
       const float w = c > 0 ? wgt(i) : -wgt(i);
-      s[d] = fma2(pair_of(w), dr, s[d]);
       if (PC)
-        sab[d] = fma2(pair_of(w), da, sab[d]);
+        A[d] = fma2(pair_of(w), make_float2(da1, da2), A[d]);
       else
-        sa[d] = __fmaf_rn(w, da1, sa[d]);
+        A[d].x = __fmaf_rn(w, da1, A[d].x);
     }
   }
+  if (!PC)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) A[d].y = A[d].x;
+}
+template <bool PC, typename RS>
+__device__ __forceinline__ void force_per_mass(const StepParams &p, const RS &rs,
+                                               float rho_tot, float2 (&gf)[3]) {
+  float2 s[3], A[3];  // (S_1, S_2) and (A_1, A_2)
+#pragma unroll
+  for (int d = 0; d < 3; ++d) s[d] = pair_of(0.0f);
+#pragma unroll
+  for (int i = 1; i <= 9; ++i) {
+    const float2 dr = sub2(rs.at(cx(i), cy(i), cz(i)), rs.at(-cx(i), -cy(i), -cz(i)));
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int c = d == 0 ? cx(i) : d == 1 ? cy(i) : cz(i);
+      if (c != 0) s[d] = fma2(pair_of(c > 0 ? wgt(i) : -wgt(i)), dr, s[d]);
+    }
+  }
+  rs.template adhesion<PC>(A);
   const float inv_rho = 1.0f / rho_tot;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    const float a1 = PC ? sab[d].x : sa[d], a2 = PC ? sab[d].y : sa[d];
-    gf[d].x = __fmaf_rn(p.F[d], inv_rho, __fmaf_rn(-p.G, s[d].y, a1));
-    gf[d].y = __fmaf_rn(p.F[d], inv_rho, __fmaf_rn(-p.G, s[d].x, -a2));
+    gf[d].x = __fmaf_rn(p.F[d], inv_rho, __fmaf_rn(-p.G, s[d].y, A[d].x));
+    gf[d].y = __fmaf_rn(p.F[d], inv_rho, __fmaf_rn(-p.G, s[d].x, -A[d].y));
   }
+}
+
+template <bool PC>
+__device__ __forceinline__ void GlobalRho::adhesion(float2 (&A)[3]) const {
+  adhesion_sum<PC>(*this, A);
 }
 
 // Reservoir face holding node (x, y, z), -1 if none; the higher face wins.
@@ -295,6 +314,17 @@ __device__ __forceinline__ void reservoir_state(const StepParams &p, bool maybe,
   }
 }
 
+// The stored form of the pair o of direction i, its destination's density
+// being dest (used by the *_LOCAL storages).
+template <int ST>
+__device__ __forceinline__ typename Codec2<ST>::T2 encode(const StepParams &p, int i, float2 o,
+                                                          float2 dest) {
+  if constexpr (storage_local(ST))
+    return Codec2<ST>::enc_local(o, wgt(i), dest);
+  else
+    return Codec2<ST>::enc(o, p.nref[wclass(i)]);
+}
+
 // Store the post-collision pair (both components) of direction i; it
 // becomes the pair of direction i of node x + c_i at t + 1.  Encoding
 // reference: w_i times the destination's density at this step (*_LOCAL;
@@ -306,11 +336,9 @@ __device__ __forceinline__ void put2(const StepParams &p, const Workspace &w,
                                      float2 rho) {
   using C = Codec2<ST>;
   typename C::T2 *f = static_cast<typename C::T2 *>(w.f);
-  typename C::T2 e;
-  if constexpr (storage_local(ST))
-    e = C::enc_local(o, wgt(i), i == 0 ? rho : rs.late(cx(i), cy(i), cz(i)));
-  else
-    e = C::enc(o, p.nref[wclass(i)]);
+  float2 dest = rho;  // the destination's density at this step (*_LOCAL)
+  if (storage_local(ST) && i != 0) dest = rs.late(cx(i), cy(i), cz(i));
+  const typename C::T2 e = encode<ST>(p, i, o, dest);
   const int slot = PARITY == 0 ? opp(i) : i;
   typename C::T2 *dst = f + (PARITY == 0 ? g.pop_off(0, 0, 0) : g.pop_off(cx(i), cy(i), cz(i)));
   if (!kChecked ||
@@ -370,42 +398,13 @@ struct Relax {
   }
 };
 
-template <int PARITY, int ST, typename RS, bool CS = false, typename GE>
-__device__ __forceinline__ void collide_put2(const StepParams &p, const Workspace &w,
-                                             const GE &g, const RS &rs,
-                                             const float2 (&v)[kQ], float2 rho,
-                                             const float2 (&u)[3], float2 ns) {
-  Relax c(make_float2(p.omega[0], p.omega[1]), ns, rho, u);
-#pragma unroll
-  for (int i = 1; i <= 9; ++i) {
-    // of the two, j = i + 9 has the positive first nonzero component, so
-    // c_j . u starts without a negation
-    const int j = i + 9;
-    float2 cu = pair_of(0.0f);
-    bool first = true;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const int c = d == 0 ? cx(j) : d == 1 ? cy(j) : cz(j);
-      if (c == 0) continue;
-      cu = first ? u[d] : (c > 0 ? add2(cu, u[d]) : sub2(cu, u[d]));
-      first = false;
-    }
-    float2 oi, oj;
-    c.pair(wclass(i) == 1, cu, v[j], v[i], oj, oi);
-    put2<PARITY, ST, RS, CS>(p, w, g, rs, i, oi, rho);
-    put2<PARITY, ST, RS, CS>(p, w, g, rs, j, oj, rho);
-  }
-  put2<PARITY, ST, RS, CS>(p, w, g, rs, 0, c.rest(v[0]), rho);
-}
-
-// Moments, forces, equilibrium velocity and collision of one node, given
-// where its neighbours' slots lie (g: pop_off) and where the step's densities
-// are found.  collide_loaded starts from the node's 19 pairs already decoded
-// (and replaced by the prescribed state inside a reservoir) and its n_s.
-template <int PARITY, int ST, bool PC, typename RS, bool CS = false, typename GE>
-__device__ __forceinline__ void collide_loaded(const StepParams &p, const Workspace &w,
-                                               const GE &g, const RS &rs,
-                                               const float2 (&v)[kQ], float2 ns) {
+// Moments, forces, equilibrium velocity and collision of one node from its
+// 19 pairs v (decoded, and replaced by the prescribed state inside a
+// reservoir), its n_s and where the step's densities are found; emit(i, o,
+// rho) takes the post-collision pair of direction i.
+template <bool PC, typename RS, typename Emit>
+__device__ __forceinline__ void collide_core(const StepParams &p, const RS &rs,
+                                             const float2 (&v)[kQ], float2 ns, Emit emit) {
   const float2 rho = sum19(v);
   float2 j[3];
   first_moment(v, j);
@@ -424,7 +423,38 @@ __device__ __forceinline__ void collide_loaded(const StepParams &p, const Worksp
     u[d].y = __fmaf_rn(jc, inv_den, __fmul_rn(p.tau[1], gf[d].y));
   }
 
-  collide_put2<PARITY, ST, RS, CS>(p, w, g, rs, v, rho, u, ns);
+  Relax c(make_float2(p.omega[0], p.omega[1]), ns, rho, u);
+#pragma unroll
+  for (int i = 1; i <= 9; ++i) {
+    // of the two, j = i + 9 has the positive first nonzero component, so
+    // c_j . u starts without a negation
+    const int k = i + 9;
+    float2 cu = pair_of(0.0f);
+    bool first = true;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int e = d == 0 ? cx(k) : d == 1 ? cy(k) : cz(k);
+      if (e == 0) continue;
+      cu = first ? u[d] : (e > 0 ? add2(cu, u[d]) : sub2(cu, u[d]));
+      first = false;
+    }
+    float2 oi, ok;
+    c.pair(wclass(i) == 1, cu, v[k], v[i], ok, oi);
+    emit(i, oi, rho);
+    emit(k, ok, rho);
+  }
+  emit(0, c.rest(v[0]), rho);
+}
+
+// The same, each pair stored where the AA pattern puts it: g tells where the
+// neighbours' slots lie (pop_off).
+template <int PARITY, int ST, bool PC, typename RS, bool CS = false, typename GE>
+__device__ __forceinline__ void collide_loaded(const StepParams &p, const Workspace &w,
+                                               const GE &g, const RS &rs,
+                                               const float2 (&v)[kQ], float2 ns) {
+  collide_core<PC>(p, rs, v, ns, [&](int i, float2 o, float2 rho) {
+    put2<PARITY, ST, RS, CS>(p, w, g, rs, i, o, rho);
+  });
 }
 
 // n_s,1 and n_s,2 (the same without per-component fractions) of a node.
@@ -515,6 +545,10 @@ struct SmemStencil {
   }
   __device__ __forceinline__ float a2(int dx, int dy, int dz) const {
     return b[dz + 1][dy * kPipeRingCols + c + dx];
+  }
+  template <bool PC>
+  __device__ __forceinline__ void adhesion(float2 (&A)[3]) const {
+    adhesion_sum<PC>(*this, A);
   }
 };
 __host__ __device__ constexpr Shape pipe_shape(int parity, bool local, int cfg) {
@@ -1285,6 +1319,10 @@ struct RingRho {
   }
   __device__ __forceinline__ float a2(int dx, int dy, int dz) const {
     return glob->a2(dx, dy, dz);
+  }
+  template <bool PC>
+  __device__ __forceinline__ void adhesion(float2 (&A)[3]) const {
+    adhesion_sum<PC>(*this, A);
   }
 };
 

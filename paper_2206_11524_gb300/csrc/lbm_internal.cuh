@@ -369,6 +369,8 @@ constexpr double kWaveSetL2Share = 0.5;
   cudaError_t launch_wave_##SUF(const StepParams &, const Workspace &, int,     \
                                 int, int, unsigned, long long, cudaStream_t);  \
   cudaError_t launch_wave_batch_##SUF(const WaveJob &, cudaStream_t);         \
+  cudaError_t launch_resident_##SUF(const StepParams &, const Workspace &, int, int, \
+                                    unsigned, bool, cudaStream_t);            \
   cudaError_t launch_batch_density_##SUF(const BatchArgs &, cudaStream_t);     \
   cudaError_t launch_batch_collide_##SUF(const BatchArgs &, cudaStream_t);     \
   cudaError_t launch_batch_collide_pipe_##SUF(const BatchArgs &, int, int, cudaStream_t);
@@ -413,6 +415,17 @@ cudaError_t launch_wave(const StepParams &p, const Workspace &w, int parity,
                         int cfg, int lag, unsigned spin_limit, long long hold,
                         cudaStream_t s);
 cudaError_t launch_wave_batch(const WaveJob &job, int storage, cudaStream_t s);
+// `steps` whole steps of a lattice of at most kResidentTiles x-tiles in one
+// launch (lbm_resident.cuh), the first at AA parity `parity`; the reservoirs
+// of p hold in all of them.  spin_limit bounds the polls of one wait of the
+// cooperative variant; hold: that variant's first barrier never completes
+// (tests of the failure path).  Leaves the last step's densities in the
+// buffer that step wrote (w.rho, or w.rho_enc after an even number of steps
+// of a local storage).  kResidentSteps bounds one launch, so that it never
+// holds its SMs for more than a few milliseconds.
+constexpr int kResidentTiles = 4608, kResidentSteps = 256;
+cudaError_t launch_resident(const StepParams &p, const Workspace &w, int parity, int steps,
+                            unsigned spin_limit, bool hold, cudaStream_t s);
 cudaError_t launch_reduce(const StepParams &p, const Workspace &w,
                           cudaStream_t s);
 

@@ -225,6 +225,17 @@ cudaError_t launch_wave(const StepParams &p, const Workspace &w, int parity,
   }
 }
 
+cudaError_t launch_resident(const StepParams &p, const Workspace &w, int parity, int steps,
+                            unsigned spin_limit, bool hold, cudaStream_t s) {
+  switch (p.storage) {
+    case kF16: return launch_resident_f16(p, w, parity, steps, spin_limit, hold, s);
+    case kBF16: return launch_resident_bf16(p, w, parity, steps, spin_limit, hold, s);
+    case kF16L: return launch_resident_f16l(p, w, parity, steps, spin_limit, hold, s);
+    case kBF16L: return launch_resident_bf16l(p, w, parity, steps, spin_limit, hold, s);
+    default: return launch_resident_f32(p, w, parity, steps, spin_limit, hold, s);
+  }
+}
+
 cudaError_t launch_wave_batch(const WaveJob &job, int storage, cudaStream_t s) {
   switch (storage) {
     case kF16: return launch_wave_batch_f16(job, s);

@@ -3,6 +3,7 @@
 // StorageKind) and HMCSC_SUF (the name suffix) defined.
 #include <mutex>
 
+#include "lbm_resident.cuh"
 #include "lbm_wave.cuh"
 
 #define HMCSC_CAT2(a, b) a##_##b
@@ -160,6 +161,95 @@ cudaError_t HMCSC_NAME(launch_single_pass)(const StepParams &p, const Workspace 
   if (w.ns2)
     return parity == 0 ? single_pass<0, true>(p, w, nzc, s) : single_pass<1, true>(p, w, nzc, s);
   return parity == 0 ? single_pass<0, false>(p, w, nzc, s) : single_pass<1, false>(p, w, nzc, s);
+}
+
+namespace {
+// Clusters of 16 blocks need a device attribute and 16 free SMs of one
+// processing cluster; *ok says whether one fits on this device at all.
+template <bool PC>
+cudaError_t cluster_config(const StepParams &p, cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr,
+                           bool *ok) {
+  using Tile = ClusterTile<typename Codec2<kST>::T2>;
+  static std::once_flag once[16];
+  static bool fits[16];
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 16) return cudaErrorInvalidDevice;
+  // as many blocks as there can be: a warp alone on its scheduler is fastest
+  // (500 nodes: 1.3 us a step in 16 blocks of a warp, 1.7 in 2 of eight)
+  auto shape = [&](int warps, int blocks) {
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)blocks;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kTile, warps, 1);
+    cfg.dynamicSmemBytes = sizeof(Tile) * warps;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+  };
+  std::call_once(once[dev], [&] {
+    auto kern = k_cluster<kST, PC>;
+    int n = 0;
+    shape(kClusterWarps, kClusterBlocks);
+    fits[dev] =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(Tile) * kClusterWarps) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n >= 1;
+    if (!fits[dev]) cudaGetLastError();  // the workspace variant takes over
+  });
+  int warps = 1;
+  while (p.ntiles > (long long)warps * kClusterBlocks) warps *= 2;
+  shape(warps, (int)((p.ntiles + warps - 1) / warps));
+  *ok = fits[dev];
+  return cudaSuccess;
+}
+template <bool PC>
+cudaError_t resident_launch(const StepParams &p, const Workspace &w, int parity, int steps,
+                            unsigned spin_limit, bool hold, cudaStream_t s) {
+  cudaLaunchAttribute attr[1];
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = s;
+  if (p.ntiles <= kClusterTiles) {
+    bool ok = false;
+    const cudaError_t e = cluster_config<PC>(p, cfg, attr[0], &ok);
+    if (e != cudaSuccess) return e;
+    if (ok) return cudaLaunchKernelEx(&cfg, k_cluster<kST, PC>, p, w, parity, steps);
+  }
+  static int sms[16];  // one block per SM (0: not asked yet)
+  static std::once_flag once[16];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 16) return cudaErrorInvalidDevice;
+  std::call_once(once[dev], [dev] {
+    cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev);
+  });
+  if (sms[dev] < 1) return cudaErrorInvalidDevice;
+  // few warps a block while that leaves SMs free (32 x 16 x 16: 4.6 us a step
+  // in 128 blocks of two warps, 5.4 in 32 of eight)
+  int warps = 1;
+  while (warps < kResidentWarps && p.ntiles > (long long)warps * sms[dev]) warps *= 2;
+  const long long blocks = (p.ntiles + warps - 1) / warps;
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.gridDim = dim3((unsigned)(blocks < sms[dev] ? blocks : sms[dev]));
+  cfg.blockDim = dim3(kTile, warps, 1);
+  cfg.dynamicSmemBytes = 0;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_resident<kST, PC>, p, w,
+                            ResidentArgs{parity, steps, spin_limit, hold ? 1 : 0});
+}
+}  // namespace
+
+cudaError_t HMCSC_NAME(launch_resident)(const StepParams &p, const Workspace &w, int parity,
+                                        int steps, unsigned spin_limit, bool hold,
+                                        cudaStream_t s) {
+  return w.ns2 ? resident_launch<true>(p, w, parity, steps, spin_limit, hold, s)
+               : resident_launch<false>(p, w, parity, steps, spin_limit, hold, s);
 }
 
 namespace {
