@@ -40,43 +40,48 @@ namespace hmcsc {
 namespace {
 
 
-// Periodic neighbourhood of one node in tile coordinates.
+// threadIdx.y and .z are the same for all lanes of a warp (blocks are 32
+// threads wide); read through lane 0 the compiler knows it too and keeps row
+// and plane arithmetic in uniform registers.
+__device__ __forceinline__ int warp_ty() { return __shfl_sync(0xffffffffu, (int)threadIdx.y, 0); }
+__device__ __forceinline__ int warp_tz() { return __shfl_sync(0xffffffffu, (int)threadIdx.z, 0); }
+
+// Periodic neighbourhood of one node: rows are uniform over a warp, the x
+// part is the lane's own.
 struct Geo {
-  int tx[3], ln[3];  // tile-x index and lane of x-1, x, x+1
-  int yw[3], zw[3];  // y-1..y+1, z-1..z+1 (wrapped)
-  int tr[3][3];      // first tile of row (y', z'): ntx * (y' + ny * z')
+  int row[3][3];     // first tile of row (y + dy, z + dz): ntx * (y' + ny * z')
+  int xw[3];         // x - 1, x, x + 1 (wrapped): the node inside its row
+  unsigned xp[3];    // pair offset of slot 0 of that node inside its row
   __device__ __forceinline__ int tile(int dx, int dy, int dz) const {
-    return tr[dy + 1][dz + 1] + tx[dx + 1];
+    return row[dy + 1][dz + 1] + xw[dx + 1] / kTile;
   }
+  __device__ __forceinline__ int lane(int dx) const { return xw[dx + 1] % kTile; }
   // tiled node index of x + (dx, dy, dz)
   __device__ __forceinline__ int node(int dx, int dy, int dz) const {
-    return tile(dx, dy, dz) * kTile + ln[dx + 1];
+    return row[dy + 1][dz + 1] * kTile + xw[dx + 1];
   }
   // pair offset of slot 0 of node x + (dx, dy, dz) in the population array
   // (fits 32 bits: the host requires ntiles * 1216 < 2^32)
   __device__ __forceinline__ unsigned pop_off(int dx, int dy, int dz) const {
-    return (unsigned)tile(dx, dy, dz) * (unsigned)kTilePairs + (unsigned)ln[dx + 1];
+    return (unsigned)row[dy + 1][dz + 1] * (unsigned)kTilePairs + xp[dx + 1];
   }
 };
 
 __device__ __forceinline__ Geo make_geo(const StepParams &p, int x, int y,
                                         int z) {
   Geo g;
-  const int xm = x == 0 ? p.nx - 1 : x - 1;
-  const int xp = x == p.nx - 1 ? 0 : x + 1;
-  g.tx[0] = xm / kTile; g.ln[0] = xm % kTile;
-  g.tx[1] = x / kTile;  g.ln[1] = x % kTile;
-  g.tx[2] = xp / kTile; g.ln[2] = xp % kTile;
-  g.yw[0] = y == 0 ? p.ny - 1 : y - 1;
-  g.yw[1] = y;
-  g.yw[2] = y == p.ny - 1 ? 0 : y + 1;
-  g.zw[0] = z == 0 ? p.nz - 1 : z - 1;
-  g.zw[1] = z;
-  g.zw[2] = z == p.nz - 1 ? 0 : z + 1;
+  g.xw[0] = x == 0 ? p.nx - 1 : x - 1;
+  g.xw[1] = x;
+  g.xw[2] = x == p.nx - 1 ? 0 : x + 1;
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    g.xp[a] = (unsigned)(g.xw[a] / kTile) * (unsigned)kTilePairs + (unsigned)(g.xw[a] % kTile);
+  const int yw[3] = {y == 0 ? p.ny - 1 : y - 1, y, y == p.ny - 1 ? 0 : y + 1};
+  const int zw[3] = {z == 0 ? p.nz - 1 : z - 1, z, z == p.nz - 1 ? 0 : z + 1};
 #pragma unroll
   for (int a = 0; a < 3; ++a)
 #pragma unroll
-    for (int b = 0; b < 3; ++b) g.tr[a][b] = p.ntx * (g.yw[a] + p.ny * g.zw[b]);
+    for (int b = 0; b < 3; ++b) g.row[a][b] = p.ntx * (yw[a] + p.ny * zw[b]);
   return g;
 }
 
@@ -598,8 +603,8 @@ __device__ __forceinline__ bool block_in_reservoir(const StepParams &p) {
 template <int BY, int BZ>
 __device__ __forceinline__ void block_coords(int &x, int &y, int &z) {
   x = blockIdx.x * kTile + threadIdx.x;
-  y = blockIdx.y * BY + threadIdx.y;
-  z = blockIdx.z * BZ + threadIdx.z;
+  y = blockIdx.y * BY + (BY > 1 ? warp_ty() : 0);
+  z = blockIdx.z * BZ + (BZ > 1 ? warp_tz() : 0);
 }
 
 template <int PARITY, int ST, int CFG>
@@ -758,21 +763,21 @@ struct RowCopy {
 // Where a block that walks along z finds a node's neighbours: the in-plane
 // part does not change from plane to plane.
 struct MarchGeo {
-  unsigned pin[3][3];  // pair offset of slot 0 of (x + dx, y + dy) inside a plane
-  unsigned pz[3];      // pair offset of planes z - 1, z, z + 1
+  unsigned row[3];     // pair offset of row y + dy inside a plane (uniform)
+  unsigned xp[3];      // pair offset of slot 0 of x + dx inside a row
+  unsigned pz[3];      // pair offset of planes z - 1, z, z + 1 (uniform)
   unsigned plane, total;
   __device__ __forceinline__ MarchGeo(const StepParams &p, int x, int y, int z) {
     plane = (unsigned)(p.ny * p.ntx) * (unsigned)kTilePairs;
     total = plane * (unsigned)p.nz;
 #pragma unroll
-    for (int b = 0; b < 3; ++b)
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        int xw = x + a - 1, yw = y + b - 1;
-        xw = xw < 0 ? p.nx - 1 : (xw >= p.nx ? 0 : xw);
-        yw = yw < 0 ? p.ny - 1 : (yw >= p.ny ? 0 : yw);
-        pin[a][b] = (unsigned)(yw * p.ntx + xw / kTile) * (unsigned)kTilePairs + xw % kTile;
-      }
+    for (int a = 0; a < 3; ++a) {
+      int xw = x + a - 1, yw = y + a - 1;
+      xw = xw < 0 ? p.nx - 1 : (xw >= p.nx ? 0 : xw);
+      yw = yw < 0 ? p.ny - 1 : (yw >= p.ny ? 0 : yw);
+      xp[a] = (unsigned)(xw / kTile) * (unsigned)kTilePairs + (unsigned)(xw % kTile);
+      row[a] = (unsigned)(yw * p.ntx) * (unsigned)kTilePairs;
+    }
     pz[1] = (unsigned)z * plane;
     pz[0] = z == 0 ? total - plane : pz[1] - plane;
     pz[2] = z == p.nz - 1 ? 0u : pz[1] + plane;
@@ -784,7 +789,7 @@ struct MarchGeo {
     pz[2] = min(o, o - total);
   }
   __device__ __forceinline__ unsigned pop_off(int dx, int dy, int dz) const {
-    return pz[dz + 1] + pin[dx + 1][dy + 1];
+    return (pz[dz + 1] + row[dy + 1]) + xp[dx + 1];
   }
 };
 
@@ -823,8 +828,8 @@ __device__ __forceinline__ void pipe_block(const StepParams &p, const Workspace 
   using Smem = PipeSmem<PARITY, ST, PC, CFG>;
   extern __shared__ __align__(16) unsigned char pipe_smem[];
   Smem &sm = *reinterpret_cast<Smem *>(pipe_smem);
-  const int tid = threadIdx.y * kTile + threadIdx.x;
-  const int x = bx * kTile + threadIdx.x, y = by0 * S.by + threadIdx.y;
+  const int ty = warp_ty(), tid = ty * kTile + threadIdx.x;
+  const int x = bx * kTile + threadIdx.x, y = by0 * S.by + ty;
   const int z0 = bz * zc, zend = min(z0 + zc, p.nz);
   const int xlo = bx * kTile, ylo = by0 * S.by;
   const bool maybe_res = box_in_reservoir(p, xlo, min(xlo + kTile, p.nx) - 1, ylo,
@@ -842,7 +847,7 @@ __device__ __forceinline__ void pipe_block(const StepParams &p, const Workspace 
   int own = ((z0 * p.ny + (row ? y : 0)) * p.ntx + bx) * kTile + threadIdx.x;
   auto prefetch = [&](int b, int n) {
     if (!row) return;
-    copy.next(w, sm.pop[b][threadIdx.y]);
+    copy.next(w, sm.pop[b][ty]);
     if (kChecked && !in_bounds(w.fault, n, nodes, kFaultGeometry)) n = 0;
     cp_async(&sm.ns[b][tid], &w.ns[n]);
     if (PC) cp_async(&sm.ns2[PC ? b : 0][PC ? tid : 0], &w.ns2[n]);
@@ -904,7 +909,7 @@ __device__ __forceinline__ void pipe_block(const StepParams &p, const Workspace 
     else
       __syncwarp();      // and every lane's
     if (active) {
-      const T2 *buf = sm.pop[b][threadIdx.y];
+      const T2 *buf = sm.pop[b][ty];
       const float2 own_prev = L ? sm.enc[L ? b : 0][L ? tid : 0] : make_float2(0.f, 0.f);
       const float ns1 = sm.ns[b][tid];
       const float2 ns = make_float2(ns1, PC ? sm.ns2[PC ? b : 0][PC ? tid : 0] : ns1);
@@ -917,7 +922,7 @@ __device__ __forceinline__ void pipe_block(const StepParams &p, const Workspace 
         collide_loaded<PARITY, ST, PC, GlobalRho, S.cs>(p, w, mg, global_rho(p, w, g), v, ns);
       } else {
         SmemStencil st;
-        const int r = threadIdx.y + 1;
+        const int r = ty + 1;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
           const int sd = slot + d < kPipeRingPlanes ? slot + d : slot + d - kPipeRingPlanes;

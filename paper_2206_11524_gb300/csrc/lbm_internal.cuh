@@ -105,7 +105,14 @@ template <> struct Codec2<kF16> {
   using T2 = __half2;
   static constexpr float kScale = kHalfScale;
   static __device__ __forceinline__ float2 dec(T2 v, float2 r) {
-    return fma2(__half22float2(v), pair_of(kHalfUnscale), r);
+    // h 2^-14 + r in one mixed operation per value: the half product is exact
+    // in float32, so it rounds as the float32 fused multiply-add does
+    const unsigned u = *reinterpret_cast<const unsigned *>(&v);
+    float2 f;
+    asm("{.reg .f16 a, b, k;\n mov.b32 {a, b}, %2;\n mov.b16 k, 0x0400;\n"
+        " fma.rn.f32.f16 %0, a, k, %3;\n fma.rn.f32.f16 %1, b, k, %4;}"
+        : "=f"(f.x), "=f"(f.y) : "r"(u), "f"(r.x), "f"(r.y));
+    return f;
   }
   static __device__ __forceinline__ T2 enc(float2 f, float2 nrs) {
     const float2 o = fma2(f, pair_of(kHalfScale), nrs);
@@ -116,7 +123,12 @@ template <> struct Codec2<kBF16> {
   using T2 = __nv_bfloat162;
   static constexpr float kScale = 1.0f;
   static __device__ __forceinline__ float2 dec(T2 v, float2 r) {
-    return add2(r, __bfloat1622float2(v));
+    const unsigned u = *reinterpret_cast<const unsigned *>(&v);
+    float2 f;
+    asm("{.reg .b16 a, b;\n mov.b32 {a, b}, %2;\n"
+        " add.rn.f32.bf16 %0, a, %3;\n add.rn.f32.bf16 %1, b, %4;}"
+        : "=f"(f.x), "=f"(f.y) : "r"(u), "f"(r.x), "f"(r.y));
+    return f;
   }
   static __device__ __forceinline__ T2 enc(float2 f, float2 nr) {
     const float2 o = add2(f, nr);

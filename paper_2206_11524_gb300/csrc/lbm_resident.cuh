@@ -62,7 +62,7 @@ __device__ __forceinline__ bool resident_barrier(const Workspace &w, const Resid
 template <int PARITY, int ST, bool PC>
 __device__ __forceinline__ bool resident_step(const StepParams &p, const Workspace &w,
                                               const ResidentArgs &a, unsigned &target, bool &ok) {
-  const int first = blockIdx.x * blockDim.y + threadIdx.y;
+  const int first = blockIdx.x * blockDim.y + warp_ty();
   const int stride = gridDim.x * blockDim.y;
   const int tiles = (int)p.ntiles;
   float2 v[kQ];
@@ -289,14 +289,14 @@ __global__ void __launch_bounds__(kTile * kClusterWarps, 1)
     const unsigned base = (unsigned)__cvta_generic_to_shared(tiles);
 #pragma unroll
     for (int d = 0; d < 3; ++d)
-      nb.to_rho[d] = (unsigned)(sizeof(T2) * kTilePairs) + g.ln[d] * (unsigned)(8 - sizeof(T2));
+      nb.to_rho[d] = (unsigned)(sizeof(T2) * kTilePairs) + g.lane(d - 1) * (unsigned)(8 - sizeof(T2));
 #pragma unroll
     for (int i = 0; i < kQ; ++i) {
       int n = g.tile(cx(i), cy(i), cz(i));
       if (!in_bounds(w.fault, n, p.ntiles, kFaultShared)) n = 0;
       nb.addr[1 + cx(i)][1 + cy(i)][1 + cz(i)] =
           cluster_map(base + (unsigned)(n % W) * (unsigned)sizeof(Tile) +
-                          g.ln[1 + cx(i)] * (unsigned)sizeof(T2),
+                          g.lane(cx(i)) * (unsigned)sizeof(T2),
                       (unsigned)(n / W));
     }
   }
