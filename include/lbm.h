@@ -173,8 +173,9 @@ LBM_API lbm_status lbm_set_bc_velocity(lbm_ctx *ctx, int face, int layers,
  * lbm_set_wavefront enabled it.  A small lattice (up to 4,608 x-tiles: nx /
  * 32, rounded up, times ny nz) without those two settings and without launch
  * shapes of the caller's (lbm_set_launch_config) takes up to 256 steps per
- * launch instead, with the same results bit for bit; its waits are bounded
- * like the wavefront's.  n_steps = 0 is a no-op.  EINTERNAL (and
+ * launch instead, and a larger float32 lattice whose planes in flight stay in
+ * L2 takes the wavefront launch with a lag of the library's choice, with the
+ * same results bit for bit; all waits are bounded like the wavefront's.  n_steps = 0 is a no-op.  EINTERNAL (and
  * nothing enqueued) when a device fault was reported for the current state:
  * by a synchronising call (below), or by a launch that already ran, through
  * a host-mapped word the kernel sets (no stream wait). */
@@ -191,8 +192,8 @@ LBM_API lbm_status lbm_step(lbm_ctx *ctx, int n_steps);
  * lbm_collide_stream and the batched entry points keep the two passes. */
 LBM_API lbm_status lbm_set_single_pass(lbm_ctx *ctx, int planes);
 
-/* Wavefront stepping for lbm_step (shape > 0; 0 = two passes, the default;
- * it takes precedence over lbm_set_single_pass): each step is one persistent
+/* Wavefront stepping for lbm_step (shape > 0; 0, the default, leaves the step
+ * to lbm_step; it takes precedence over lbm_set_single_pass): each step is one persistent
  * cooperative launch over work items, a tile of 32 x by nodes of one plane
  * each (shape 1: by = 4, 2: by = 2, 3: by = 8), taken in plane order from an
  * atomic ticket.  An item sums the populations of one plane's tile into the

@@ -42,6 +42,8 @@ struct lbm_ctx {
   uint64_t bc_version;    // bumped by every lbm_set_bc
   int launch_cfg[3];      // launch shapes: density, even fused, odd fused
   bool launch_cfg_set;    // by the caller: lbm_step keeps the passes they are for
+  int auto_lag;           // wave_auto_lag: > 0: lbm_step's own choice is the
+                          // wavefront launch with this lag
   int single_pass_zc;     // > 0: lbm_step sweeps once, boxes of this many planes
   int wave_cfg;           // > 0: lbm_step is one wavefront launch of this shape
   int wave_lag;           // planes between a plane's density and its collision
@@ -372,6 +374,7 @@ lbm_status lbm_create(const lbm_params *params, void *d_workspace,
   c->launch_cfg[1] = f32 ? 6 : 9;
   c->launch_cfg[2] = f32 ? 7 : local ? 9 : 8;
   c->launch_cfg_set = false;
+  c->auto_lag = hmcsc::wave_auto_lag(sp);
   c->single_pass_zc = 0;
   c->wave_cfg = 0;
   c->wave_lag = hmcsc::kWaveLagDefault;
@@ -687,9 +690,14 @@ lbm_status lbm_step(lbm_ctx *c, int n_steps) {
       k += m - 1;
       continue;
     }
-    if (c->wave_cfg > 0) {
-      cudaError_t e = hmcsc::launch_wave(c->sp, c->ws, parity(c), c->wave_cfg, c->wave_lag,
-                                         c->wave_spin, c->wave_hold, c->stream);
+    // the wavefront launch, asked for or chosen (for a lattice whose caller
+    // asked for no step in particular)
+    const bool own_choice =
+        c->wave_cfg == 0 && c->single_pass_zc == 0 && !c->launch_cfg_set && c->auto_lag > 0;
+    if (c->wave_cfg > 0 || own_choice) {
+      cudaError_t e = hmcsc::launch_wave(c->sp, c->ws, parity(c), own_choice ? 2 : c->wave_cfg,
+                                         own_choice ? c->auto_lag : c->wave_lag, c->wave_spin,
+                                         c->wave_hold, c->stream);
       if (e != cudaSuccess) return cuda_fail(c, e, "wavefront kernel");
       c->rho_at = c->t;
       finish_step(c);

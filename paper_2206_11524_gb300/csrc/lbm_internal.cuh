@@ -297,6 +297,36 @@ __host__ __device__ inline long long wave_flag_words(long long nx, long long ny,
 
 constexpr int kSms = 152;        // SMs of a GB300
 constexpr int kRedBlocks = 2 * kSms;
+
+// Lag with which a lattice that asks for no particular step takes the
+// wavefront launch (tiles of 32 x 2), 0 where the two passes are faster.
+//
+// Lag.  8 blocks per SM hold 1,216 items at a time, and a collision needs the
+// densities of two groups of tiles fewer than lag back, so the launch starves
+// unless (lag - 2) groups are well over what is in flight; every plane more
+// costs L2.  Measured for (lag - 2) x tiles per plane, us a step: 128^3 1,536
+// 245, 2,048 143, 2,560 144, 4,096 157; 192^3 1,728 586, 2,304 455, 2,880 474;
+// 224^3 1,568 1,141, 2,352 726, 3,136 772; 256^3 1,024 2,581, 2,048 1,103,
+// 3,072 1,165.  Hence the least lag that reaches 2,040.
+//
+// Where it wins (two passes, wavefront, us a step): 96^3 73.2, 68.4; 128^3
+// 168, 143; 150 x 90 x 70 81, 75; 160^3 319, 268; 192^3 524, 455; 224^3 822,
+// 726; 400 x 100 x 300 885, 792; 256^3 1,210, 1,103; 288^3 1,718, 1,646
+// (76 MB of planes in flight); 320^3 2,347, 2,362 (93 MB); 512 x 512 x 100
+// 1,878, 1,982 -- while lag + 2 planes stay in L2.  A launch runs nz + lag
+// groups, so short lattices lose: nz of five lags at least.  The 16-bit
+// storages stay with two passes, whose stencil comes from shared memory
+// (128^3 half offsets 107, 132).
+inline int wave_auto_lag(const StepParams &p) {
+  constexpr double kL2Planes = 80e6;  // bytes of planes in flight
+  constexpr long long kAhead = 2040;  // items: 1.7 times what is in flight
+  if (p.storage != kF32) return 0;
+  const long long tp = (long long)p.ntx * ((p.ny + 1) / 2);
+  const long long lag = 2 + (kAhead + tp - 1) / tp;
+  const double plane = (double)p.ntx * kTile * p.ny * kQ * sizeof(float2);
+  if (p.nz < 5 * lag || (double)(lag + 2) * plane > kL2Planes) return 0;
+  return (int)lag;
+}
 constexpr int kRedThreads = 256;
 constexpr int kRedK = 11;        // mass[2], sat num/den, p_face[6], nonfinite
 
