@@ -50,7 +50,7 @@ struct lbm_ctx {
   uint32_t wave_spin;     // polls of one flag before a wavefront wait gives up
   int64_t wave_hold;      // flag the warp-item launch leaves unpublished (-1)
   unsigned *fault_host;   // host-mapped word set by a wait that ran out, or NULL
-  int fault_slot;         // its slot in the process-wide page (-1: none)
+  int fault_slot;         // its slot among the process-wide ones (-1: none)
   bool fault_seen;        // a device fault was reported for the current state
   std::string err;
 };
@@ -66,29 +66,49 @@ struct lbm_graph {
 
 namespace {
 
-// Host-mapped fault words, one per context, from one pinned page allocated
-// once per process (allocating and freeing pinned memory per context would
-// synchronise the device every time a context is destroyed).
+// Host-mapped memory that kernels write results into, allocated once per
+// process (allocating and freeing pinned memory per context would synchronise
+// the device every time a context is destroyed): a slot per context -- the
+// fault word on a 64-byte line of its own, then what the reductions return --
+// and one buffer through which small read-backs pass.  A kernel that writes
+// there replaces its copies: a copy of a few bytes to pageable memory costs
+// about 15 us with its own wait, and six more to the fields' arrays 20 us.
 constexpr int kFaultSlots = 4096;
+struct HostSlot {
+  unsigned fault;                     // set by a wait that ran out
+  unsigned word;                      // copy of the workspace's fault word
+  unsigned pad[14];
+  hmcsc::ReduceResult reduce;
+  unsigned char pad2[192 - sizeof(hmcsc::ReduceResult)];
+};
+static_assert(sizeof(HostSlot) == 256, "a slot is four lines");
+// What may pass through the buffer: the host copies it out once more (about
+// 12 GB/s), so the six copies of the fields win from some 200 KB on (32 x 16 x
+// 16, 196 KB: 48 us either way; six lattices of 32^3 .. 48^3: 0.36 ms by
+// copies, 0.82 through the buffer) and the staged rounds of the populations,
+// seven launches and copies, from some 1 MB on.
+constexpr size_t kBounceBytes = 1u << 20, kBounceFields = 128u << 10;
 std::mutex g_fault_mu;
-unsigned *g_fault_host = nullptr;     // host view of the page
-unsigned *g_fault_dev = nullptr;      // its device view
+HostSlot *g_fault_host = nullptr;     // host view
+HostSlot *g_fault_dev = nullptr;      // device view
+std::mutex g_bounce_mu;               // held from the launch to the last byte taken out
 bool g_fault_tried = false;
 std::vector<int> g_fault_free;
 
 // A slot's host and device pointers, or false when mapped host memory is
-// unavailable or every slot is taken (the synchronising checks remain).
-bool fault_slot_take(unsigned **host, unsigned **dev, int *slot) {
+// unavailable or every slot is taken (copies and waits do then).
+bool fault_slot_take(HostSlot **host, HostSlot **dev, int *slot) {
   std::lock_guard<std::mutex> lock(g_fault_mu);
   if (!g_fault_tried) {
     g_fault_tried = true;
     void *h = nullptr, *d = nullptr;
-    if (cudaHostAlloc(&h, kFaultSlots * 16 * sizeof(unsigned), cudaHostAllocMapped) ==
+    const size_t slots = kFaultSlots * sizeof(HostSlot);
+    if (cudaHostAlloc(&h, slots + kBounceBytes, cudaHostAllocMapped | cudaHostAllocPortable) ==
         cudaSuccess) {
       if (cudaHostGetDevicePointer(&d, h, 0) == cudaSuccess) {
-        memset(h, 0, kFaultSlots * 16 * sizeof(unsigned));
-        g_fault_host = static_cast<unsigned *>(h);
-        g_fault_dev = static_cast<unsigned *>(d);
+        memset(h, 0, slots);
+        g_fault_host = static_cast<HostSlot *>(h);
+        g_fault_dev = static_cast<HostSlot *>(d);
         for (int k = kFaultSlots - 1; k >= 0; --k) g_fault_free.push_back(k);
       } else {
         cudaFreeHost(h);
@@ -99,12 +119,24 @@ bool fault_slot_take(unsigned **host, unsigned **dev, int *slot) {
   if (!g_fault_host || g_fault_free.empty()) return false;
   *slot = g_fault_free.back();
   g_fault_free.pop_back();
-  // one word per 64-byte line, so contexts never share a line
-  *host = g_fault_host + *slot * 16;
-  *dev = g_fault_dev + *slot * 16;
-  *(volatile unsigned *)*host = 0u;
+  *host = g_fault_host + *slot;
+  *dev = g_fault_dev + *slot;
+  *(volatile unsigned *)&(*host)->fault = 0u;
   return true;
 }
+
+// The read-back buffer, for a call that needs `bytes` of it: host and device
+// views, or NULL when there is none, it is too small or another thread has it.
+struct Bounce {
+  std::unique_lock<std::mutex> lock;
+  char *host = nullptr;
+  char *dev = nullptr;
+  Bounce(size_t bytes, size_t most) : lock(g_bounce_mu, std::defer_lock) {
+    if (!g_fault_host || bytes > most || !lock.try_lock()) return;
+    host = reinterpret_cast<char *>(g_fault_host + kFaultSlots);
+    dev = reinterpret_cast<char *>(g_fault_dev + kFaultSlots);
+  }
+};
 
 void fault_slot_give(int slot) {
   if (slot < 0) return;
@@ -160,10 +192,9 @@ size_t pop_bytes(const lbm_ctx *c) {
   return pop_floats(c) * (size_t)hmcsc::storage_bytes(c->sp.storage);
 }
 
-// Host-side encode / decode of one population in the context's storage
-// with the reference w_i rho_ref already formed (the same float operations
-// the kernels use: subtract, round to nearest into half / bfloat16; decode
-// by adding the reference back).
+// Host-side encode of one population in the context's storage with the
+// reference w_i rho_ref already formed (the same float operations the kernels
+// use: subtract, round to nearest into half / bfloat16).
 void encode(int storage, void *dst, size_t idx, float f, float ref) {
   if (storage == hmcsc::kF16 || storage == hmcsc::kF16L)
     static_cast<__half *>(dst)[idx] = __float2half_rn((f - ref) * hmcsc::kHalfScale);
@@ -171,13 +202,6 @@ void encode(int storage, void *dst, size_t idx, float f, float ref) {
     static_cast<__nv_bfloat16 *>(dst)[idx] = __float2bfloat16_rn(f - ref);
   else
     static_cast<float *>(dst)[idx] = f;
-}
-float decode(int storage, const void *src, size_t idx, float ref) {
-  if (storage == hmcsc::kF16 || storage == hmcsc::kF16L)
-    return ref + __half2float(static_cast<const __half *>(src)[idx]) * hmcsc::kHalfUnscale;
-  if (storage == hmcsc::kBF16 || storage == hmcsc::kBF16L)
-    return ref + __bfloat162float(static_cast<const __nv_bfloat16 *>(src)[idx]);
-  return static_cast<const float *>(src)[idx];
 }
 
 // Tiled node index of (x, y, z).
@@ -193,8 +217,8 @@ void set_density_views(lbm_ctx *c) {
   c->ws.rho = c->rho_buf[1 - c->enc];
 }
 
-// Reference of population i (component s) of node (x,y,z) for decoding or
-// encoding it as stored: *_LOCAL uses the node's own previous density in
+// Reference of population i (component s) of node (x,y,z) for encoding it as
+// stored: *_LOCAL uses the node's own previous density in
 // rho_enc (host copy, tiled float2), *_OFFSET the constant table.
 float stored_ref(const lbm_ctx *c, const float *rho_enc_host, int s, int i,
                  int x, int y, int z) {
@@ -215,14 +239,10 @@ size_t pop_offset(const lbm_ctx *c, int k, long long x, long long y, long long z
 
 int parity(const lbm_ctx *c) { return (int)(c->t & 1); }
 
-// The fault word after the context's stream has drained: EINTERNAL (with a
+// What the fault word says once the stream has drained: EINTERNAL (with a
 // message) when a bit is set, which also makes lbm_step refuse to advance
 // the state until it is replaced or the word cleared.
-lbm_status check_fault(lbm_ctx *c) {
-  unsigned v = 0;
-  cudaError_t e = cudaMemcpyAsync(&v, c->ws.fault, sizeof v, cudaMemcpyDeviceToHost, c->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "fault word");
+lbm_status judge_fault(lbm_ctx *c, unsigned v) {
   if (c->fault_host && *(volatile unsigned *)c->fault_host) v |= hmcsc::kFaultWait;
   if (v == 0) return LBM_OK;
   c->fault_seen = true;
@@ -232,6 +252,24 @@ lbm_status check_fault(lbm_ctx *c) {
                 "load a checkpoint or set a new state", v);
   return fail(c, LBM_EINTERNAL,
               "the bounds-checked build recorded an out-of-range access (fault word 0x%x)", v);
+}
+
+// Wait for the stream, then judge the fault word: one wait for both where the
+// word can be copied to the context's slot.  *synced: the stream has drained
+// (results copied before are there even when a fault is reported).
+lbm_status sync_and_check(lbm_ctx *c, const char *what, bool *synced) {
+  *synced = false;
+  unsigned v = 0;
+  unsigned *dst = c->fault_slot >= 0 ? &g_fault_host[c->fault_slot].word : &v;
+  cudaError_t e = cudaMemcpyAsync(dst, c->ws.fault, sizeof v, cudaMemcpyDeviceToHost, c->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+  if (e != cudaSuccess) return cuda_fail(c, e, what);
+  *synced = true;
+  return judge_fault(c, *(volatile unsigned *)dst);
+}
+lbm_status check_fault(lbm_ctx *c) {
+  bool synced;
+  return sync_and_check(c, "fault word", &synced);
 }
 
 // A new state replaces one a wavefront wait may have left undefined: the
@@ -250,19 +288,6 @@ lbm_status clear_wait_fault(lbm_ctx *c) {
   if (c->fault_host) *(volatile unsigned *)c->fault_host = 0u;
   c->fault_seen = false;
   return LBM_OK;
-}
-
-// Reservoir face of node (x, y, z) for reservoir set r (higher face wins).
-int reservoir_face(const hmcsc::Reservoirs &r, const lbm_params &p, int x,
-                   int y, int z) {
-  int face = -1;
-  if (r.layers[0] && x < r.layers[0]) face = 0;
-  if (r.layers[1] && x >= p.nx - r.layers[1]) face = 1;
-  if (r.layers[2] && y < r.layers[2]) face = 2;
-  if (r.layers[3] && y >= p.ny - r.layers[3]) face = 3;
-  if (r.layers[4] && z < r.layers[4]) face = 4;
-  if (r.layers[5] && z >= p.nz - r.layers[5]) face = 5;
-  return face;
 }
 
 // Checkpoint header.
@@ -387,11 +412,11 @@ lbm_status lbm_create(const lbm_params *params, void *d_workspace,
   c->fault_host = nullptr;
   c->fault_slot = -1;
   {
-    unsigned *h = nullptr, *d = nullptr;
+    HostSlot *h = nullptr, *d = nullptr;
     int slot = -1;
     if (fault_slot_take(&h, &d, &slot)) {
-      c->fault_host = h;
-      c->ws.fault_host = d;
+      c->fault_host = &h->fault;
+      c->ws.fault_host = &d->fault;
       c->fault_slot = slot;
     }
   }
@@ -553,55 +578,30 @@ lbm_status lbm_get_populations(lbm_ctx *c, float *f) {
   if (!c) return LBM_EINVAL;
   if (!f) return fail(c, LBM_EINVAL, "f is NULL");
   if (!c->have_state) return fail(c, LBM_ESTATE, "no state set");
-  const long long N = c->N;
-  std::vector<char> raw(pop_bytes(c));
-  cudaError_t e = cudaMemcpyAsync(raw.data(), c->ws.f, raw.size(),
-                                  cudaMemcpyDeviceToHost, c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "device-to-host copy");
-  const bool local = hmcsc::storage_local(c->sp.storage);
-  std::vector<float> rho_enc(local ? 2 * (size_t)c->sp.ntiles * hmcsc::kTile : 0);
-  if (local) {
-    e = cudaMemcpyAsync(rho_enc.data(), c->ws.rho_enc, rho_enc.size() * sizeof(float),
-                        cudaMemcpyDeviceToHost, c->stream);
+  // decoded on the device into the read-back buffer, or for larger lattices
+  // into the staging planes, as many of the 38 at a time as fit
+  const size_t plane = sizeof(float) * (size_t)c->N;
+  bool synced;
+  Bounce bounce(2 * kQ * plane, kBounceBytes);
+  if (bounce.dev) {
+    cudaError_t e = hmcsc::launch_populations(c->sp, c->ws, parity(c),
+                                              reinterpret_cast<float *>(bounce.dev), 0, 2 * kQ,
+                                              c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "populations kernel");
+    const lbm_status st = sync_and_check(c, "get_populations", &synced);
+    if (synced) memcpy(f, bounce.host, 2 * kQ * plane);
+    return st;
+  }
+  for (int k = 0; k < 2 * kQ; k += 6) {
+    const int n = 2 * kQ - k < 6 ? 2 * kQ - k : 6;
+    cudaError_t e = hmcsc::launch_populations(c->sp, c->ws, parity(c), c->ws.stage, k, n,
+                                              c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "populations kernel");
+    e = cudaMemcpyAsync(f + (size_t)k * c->N, c->ws.stage, n * plane, cudaMemcpyDeviceToHost,
+                        c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "device-to-host copy");
   }
-  lbm_status st = sync_stream(c, "get_populations");
-  if (st) return st;
-  const lbm_status fst = check_fault(c);
-  const int nx = c->params.nx, ny = c->params.ny, nz = c->params.nz;
-  for (int s = 0; s < 2; ++s)
-    for (int i = 0; i < kQ; ++i)
-      for (int z = 0; z < nz; ++z)
-        for (int y = 0; y < ny; ++y)
-          for (int x = 0; x < nx; ++x) {
-            const long long n = x + (long long)nx * (y + (long long)ny * z);
-            float v;
-            if (parity(c) == 0) {
-              v = decode(c->sp.storage, raw.data(), pop_offset(c, s * kQ + i, x, y, z),
-                         stored_ref(c, rho_enc.data(), s, i, x, y, z));
-            } else {
-              // population i of node n sits in slot opp(i) of node n - c_i
-              const int xs = (x - hmcsc::cx(i) + nx) % nx;
-              const int ys = (y - hmcsc::cy(i) + ny) % ny;
-              const int zs = (z - hmcsc::cz(i) + nz) % nz;
-              v = decode(c->sp.storage, raw.data(),
-                         pop_offset(c, s * kQ + hmcsc::opp(i), xs, ys, zs),
-                         stored_ref(c, rho_enc.data(), s, i, x, y, z));
-            }
-            if (c->sp.res.any) {
-              // a node inside a reservoir holds its prescribed equilibrium
-              // (see the kernels)
-              const int face = reservoir_face(c->sp.res, c->params, x, y, z);
-              if (face >= 0) {
-                const hmcsc::Reservoirs &r = c->sp.res;
-                v = r.moving ? hmcsc::res_feq(i, r.rho[face][s], r.u[face][0],
-                                              r.u[face][1], r.u[face][2])
-                             : hmcsc::wgt(i) * r.rho[face][s];
-              }
-            }
-            f[((size_t)s * kQ + i) * N + n] = v;
-          }
-  return fst;
+  return sync_and_check(c, "get_populations", &synced);
 }
 
 lbm_status lbm_set_bc_velocity(lbm_ctx *c, int face, int layers, double rho_a,
@@ -772,21 +772,36 @@ lbm_status lbm_read_fields(lbm_ctx *c, float *rho_a, float *rho_b, float *u,
   cudaError_t e = hmcsc::launch_density(c->sp, c->ws, parity(c), c->launch_cfg[0], c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "density kernel");
   c->rho_at = c->t;
-  e = hmcsc::launch_fields(c->sp, c->ws, parity(c), c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "fields kernel");
-  const size_t L = lin_stride(c);
   const size_t bytes = sizeof(float) * (size_t)c->N;
   float *dst[6] = {rho_a, rho_b, u, u ? u + c->N : nullptr,
                    u ? u + 2 * c->N : nullptr, p};
-  for (int k = 0; k < 6; ++k) {
-    if (!dst[k]) continue;
-    e = cudaMemcpyAsync(dst[k], c->ws.stage + (size_t)k * L, bytes,
-                        cudaMemcpyDeviceToHost, c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "device-to-host copy");
+  // small fields are written straight into host-mapped memory, packed, and
+  // need no copies; without u the densities say all
+  Bounce bounce(6 * bytes, kBounceFields);
+  hmcsc::StepParams sp = c->sp;
+  hmcsc::Workspace ws = c->ws;
+  if (bounce.dev) {
+    sp.nlin = c->N;
+    ws.stage = reinterpret_cast<float *>(bounce.dev);
   }
-  lbm_status st = sync_stream(c, "read_fields");
-  if (st) return st;
-  return check_fault(c);
+  e = u ? hmcsc::launch_fields(sp, ws, parity(c), c->stream)
+        : hmcsc::launch_density_fields(sp, ws, c->stream);
+  if (e != cudaSuccess) return cuda_fail(c, e, "fields kernel");
+  if (!bounce.dev) {
+    const size_t L = lin_stride(c);
+    for (int k = 0; k < 6; ++k) {
+      if (!dst[k]) continue;
+      e = cudaMemcpyAsync(dst[k], c->ws.stage + (size_t)k * L, bytes,
+                          cudaMemcpyDeviceToHost, c->stream);
+      if (e != cudaSuccess) return cuda_fail(c, e, "device-to-host copy");
+    }
+  }
+  bool synced;
+  const lbm_status st = sync_and_check(c, "read_fields", &synced);
+  if (synced && bounce.dev)
+    for (int k = 0; k < 6; ++k)
+      if (dst[k]) memcpy(dst[k], bounce.host + (size_t)k * bytes, bytes);
+  return st;
 }
 
 lbm_status lbm_reduce(lbm_ctx *c, lbm_observables *out) {
@@ -799,15 +814,24 @@ lbm_status lbm_reduce(lbm_ctx *c, lbm_observables *out) {
   c->rho_at = c->t;
   hmcsc::StepParams obs = c->sp;
   obs.res = c->res_current;
-  e = hmcsc::launch_reduce(obs, c->ws, c->stream);
+  // the result goes straight to the context's slot; without one it passes
+  // through the workspace
+  hmcsc::ReduceResult host, *dev;
+  if (c->fault_slot >= 0)
+    dev = &g_fault_dev[c->fault_slot].reduce;
+  else
+    dev = reinterpret_cast<hmcsc::ReduceResult *>(c->ws.stage);
+  e = hmcsc::launch_reduce(obs, c->ws, dev, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "reduce kernel");
-  double r[kRedK];
-  e = cudaMemcpyAsync(r, c->ws.red + (size_t)kRedBlocks * kRedK, sizeof r,
-                      cudaMemcpyDeviceToHost, c->stream);
-  if (e != cudaSuccess) return cuda_fail(c, e, "device-to-host copy");
+  if (c->fault_slot < 0) {
+    e = cudaMemcpyAsync(&host, dev, sizeof host, cudaMemcpyDeviceToHost, c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "device-to-host copy");
+  }
   lbm_status st = sync_stream(c, "reduce");
   if (st) return st;
-  const lbm_status fst = check_fault(c);
+  if (c->fault_slot >= 0) host = g_fault_host[c->fault_slot].reduce;
+  const lbm_status fst = judge_fault(c, host.fault);
+  const double *r = host.value;
   out->mass[0] = r[0];
   out->mass[1] = r[1];
   out->sat1 = r[3] > 0.0 ? r[2] / r[3] : NAN;

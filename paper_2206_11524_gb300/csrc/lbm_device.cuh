@@ -1009,6 +1009,30 @@ __device__ __forceinline__ long long tiled_of_linear(const StepParams &p,
   return (yz * p.ntx + x / kTile) * kTile + x % kTile;
 }
 
+// Populations k0 .. k0 + nk - 1 (k = s * 19 + i) of the current state, decoded,
+// in the natural layout: out[k - k0][n], n linear, x fastest.  Blocks as
+// k_fields.
+template <int PARITY, int ST>
+__global__ void __launch_bounds__(kTile * kFieldsBY * kFieldsBZ)
+    k_populations(StepParams p, Workspace w, float *__restrict__ out, int k0, int nk) {
+  int x, y, z;
+  block_coords<kFieldsBY, kFieldsBZ>(x, y, z);
+  const bool maybe_res = block_in_reservoir<kFieldsBY, kFieldsBZ>(p);
+  if (x >= p.nx || y >= p.ny || z >= p.nz) return;
+  const Geo g = make_geo(p, x, y, z);
+  float2 v[kQ];
+  load_pops<PARITY, ST>(p, w, g, v);
+  reservoir_state(p, maybe_res, x, y, z, v);
+  const long long N = (long long)p.nx * p.ny * p.nz;
+  const long long n = x + (long long)p.nx * (y + (long long)p.ny * z);
+#pragma unroll
+  for (int i = 0; i < kQ; ++i) {
+    const int k = i - k0, m = kQ + i - k0;
+    if (k >= 0 && k < nk) out[k * N + n] = v[i].x;
+    if (m >= 0 && m < nk) out[m * N + n] = v[i].y;
+  }
+}
+
 // f_i = w_i rho_sigma at rest.  *_LOCAL storages take the initial
 // densities as the previous densities of time 0.
 template <int ST>

@@ -404,6 +404,8 @@ constexpr double kWaveSetL2Share = 0.5;
                                    int, cudaStream_t);                         \
   cudaError_t launch_fields_##SUF(const StepParams &, const Workspace &, int,  \
                                   cudaStream_t);                               \
+  cudaError_t launch_populations_##SUF(const StepParams &, const Workspace &, int, float *, \
+                                       int, int, cudaStream_t);                         \
   cudaError_t launch_init_##SUF(const StepParams &, const Workspace &,         \
                                 const float *, const float *, cudaStream_t);   \
   cudaError_t launch_single_pass_##SUF(const StepParams &, const Workspace &,  \
@@ -468,7 +470,20 @@ cudaError_t launch_wave_batch(const WaveJob &job, int storage, cudaStream_t s);
 constexpr int kResidentTiles = 4608, kResidentSteps = 256;
 cudaError_t launch_resident(const StepParams &p, const Workspace &w, int parity, int steps,
                             unsigned spin_limit, bool hold, cudaStream_t s);
-cudaError_t launch_reduce(const StepParams &p, const Workspace &w,
+// Populations k0 .. k0 + nk - 1 (k = 19 s + i) of the current state to
+// out[nk][N] (device-accessible).
+cudaError_t launch_populations(const StepParams &p, const Workspace &w, int parity, float *out,
+                               int k0, int nk, cudaStream_t s);
+// The fields that depend on the densities alone (rho_1, rho_2 and p) from
+// w.rho into their planes of w.stage, as k_fields writes them.
+cudaError_t launch_density_fields(const StepParams &p, const Workspace &w, cudaStream_t s);
+// Observables of w.rho; the kRedK results and the fault word end in *out
+// (device-accessible).
+struct ReduceResult {
+  double value[kRedK];
+  unsigned fault;
+};
+cudaError_t launch_reduce(const StepParams &p, const Workspace &w, ReduceResult *out,
                           cudaStream_t s);
 
 }  // namespace hmcsc

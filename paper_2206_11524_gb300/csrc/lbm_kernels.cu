@@ -96,12 +96,29 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce(StepParams p,
   }
 }
 
-__global__ void k_reduce_final(Workspace w) {
+// The blocks' sums in block order (a chain of FP64 additions, 6 us for all of
+// them; the blocks past a small lattice's nodes hold zeros and are not run).
+__global__ void k_reduce_final(Workspace w, int blocks, ReduceResult *out) {
   const int k = threadIdx.x;
+  if (k == kRedK) out->fault = *(volatile unsigned *)w.fault;
   if (k >= kRedK) return;
   double t = 0.0;
-  for (int b = 0; b < kRedBlocks; ++b) t += w.red[b * kRedK + k];
-  w.red[kRedBlocks * kRedK + k] = t;
+  for (int b = 0; b < blocks; ++b) t += w.red[b * kRedK + k];
+  out->value[k] = t;
+}
+
+__global__ void k_density_fields(StepParams p, Workspace w) {
+  const long long N = (long long)p.nx * p.ny * p.nz, L = p.nlin;
+  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
+       n += (long long)gridDim.x * blockDim.x) {
+    long long tn = tiled_of_linear(p, n);
+    if (!in_bounds(w.fault, tn, p.ntiles * kTile, kFaultRhoLoad)) tn = 0;
+    const float2 r = w.rho[tn];
+    const float r1 = r.x, r2 = r.y, rho = r1 + r2;
+    w.stage[n] = r1;
+    w.stage[L + n] = r2;
+    w.stage[5 * L + n] = (rho + p.G * r1 * r2) * (1.0f / 3.0f);
+  }
 }
 
 int flat_blocks(const StepParams &p) {
@@ -281,12 +298,30 @@ cudaError_t launch_batch_collide(const BatchArgs &a, int storage, cudaStream_t s
   }
 }
 
-cudaError_t launch_reduce(const StepParams &p, const Workspace &w,
+cudaError_t launch_populations(const StepParams &p, const Workspace &w, int parity, float *out,
+                               int k0, int nk, cudaStream_t s) {
+  switch (p.storage) {
+    case kF16: return launch_populations_f16(p, w, parity, out, k0, nk, s);
+    case kBF16: return launch_populations_bf16(p, w, parity, out, k0, nk, s);
+    case kF16L: return launch_populations_f16l(p, w, parity, out, k0, nk, s);
+    case kBF16L: return launch_populations_bf16l(p, w, parity, out, k0, nk, s);
+    default: return launch_populations_f32(p, w, parity, out, k0, nk, s);
+  }
+}
+
+cudaError_t launch_density_fields(const StepParams &p, const Workspace &w, cudaStream_t s) {
+  k_density_fields<<<flat_blocks(p), 256, 0, s>>>(p, w);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_reduce(const StepParams &p, const Workspace &w, ReduceResult *out,
                           cudaStream_t s) {
-  k_reduce<<<kRedBlocks, kRedThreads, 0, s>>>(p, w);
+  const long long need = (p.ntiles * kTile + kRedThreads - 1) / kRedThreads;
+  const int blocks = (int)(need < kRedBlocks ? need : kRedBlocks);
+  k_reduce<<<blocks, kRedThreads, 0, s>>>(p, w);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_reduce_final<<<1, 32, 0, s>>>(w);
+  k_reduce_final<<<1, 32, 0, s>>>(w, blocks, out);
   return cudaGetLastError();
 }
 

@@ -125,6 +125,16 @@ cudaError_t HMCSC_NAME(launch_fields)(const StepParams &p, const Workspace &w,
   return cudaGetLastError();
 }
 
+cudaError_t HMCSC_NAME(launch_populations)(const StepParams &p, const Workspace &w, int parity,
+                                           float *out, int k0, int nk, cudaStream_t s) {
+  const dim3 grid(p.ntx, (p.ny + kFieldsBY - 1) / kFieldsBY,
+                  (p.nz + kFieldsBZ - 1) / kFieldsBZ);
+  const dim3 block(kTile, kFieldsBY, kFieldsBZ);
+  if (parity == 0) k_populations<0, kST><<<grid, block, 0, s>>>(p, w, out, k0, nk);
+  else k_populations<1, kST><<<grid, block, 0, s>>>(p, w, out, k0, nk);
+  return cudaGetLastError();
+}
+
 cudaError_t HMCSC_NAME(launch_init)(const StepParams &p, const Workspace &w,
                                     const float *rho_a, const float *rho_b,
                                     cudaStream_t s) {
