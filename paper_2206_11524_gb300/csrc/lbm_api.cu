@@ -88,6 +88,7 @@ static_assert(sizeof(HostSlot) == 256, "a slot is four lines");
 // copies, 0.82 through the buffer) and the staged rounds of the populations,
 // seven launches and copies, from some 1 MB on.
 constexpr size_t kBounceBytes = 1u << 20, kBounceFields = 128u << 10;
+constexpr size_t kDirectRagged = 4u << 20;
 std::mutex g_fault_mu;
 HostSlot *g_fault_host = nullptr;     // host view
 HostSlot *g_fault_dev = nullptr;      // device view
@@ -304,6 +305,36 @@ lbm_status sync_stream(lbm_ctx *c, const char *what) {
   cudaError_t e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, what);
   return LBM_OK;
+}
+
+// Can kernels on the current device write any host memory at its host address
+// (a coherent host link)?  Then no pointer a caller hands over can fault.
+bool pageable_access() {
+  static std::once_flag once[16];
+  static bool yes[16];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 16) return false;
+  std::call_once(once[dev], [dev] {
+    int v = 0;
+    yes[dev] = cudaDeviceGetAttribute(&v, cudaDevAttrPageableMemoryAccess, dev) == cudaSuccess &&
+               v != 0;
+  });
+  return yes[dev];
+}
+// Is the array pinned from its first byte to its last, at its host address?
+// (Kernel writes reach pinned memory at the copy engine's 193 GB/s, and the
+// six copies of small fields cost 2.5 us each.)
+bool pinned_array(const void *p, size_t bytes) {
+  const char *end[2] = {(const char *)p, (const char *)p + bytes - 1};
+  for (const char *q : end) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, q) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (at.type != cudaMemoryTypeHost || at.devicePointer != (const void *)q) return false;
+  }
+  return true;
 }
 
 // Upload n floats from host to a device staging plane (pageable copy).
@@ -775,20 +806,29 @@ lbm_status lbm_read_fields(lbm_ctx *c, float *rho_a, float *rho_b, float *u,
   const size_t bytes = sizeof(float) * (size_t)c->N;
   float *dst[6] = {rho_a, rho_b, u, u ? u + c->N : nullptr,
                    u ? u + 2 * c->N : nullptr, p};
-  // small fields are written straight into host-mapped memory, packed, and
-  // need no copies; without u the densities say all
+  // small fields are written into the read-back buffer, fields for pinned
+  // arrays straight into those, others into the staging planes, from which
+  // they are copied; without u the densities say all
   Bounce bounce(6 * bytes, kBounceFields);
-  hmcsc::StepParams sp = c->sp;
-  hmcsc::Workspace ws = c->ws;
-  if (bounce.dev) {
-    sp.nlin = c->N;
-    ws.stage = reinterpret_cast<float *>(bounce.dev);
-  }
-  e = u ? hmcsc::launch_fields(sp, ws, parity(c), c->stream)
-        : hmcsc::launch_density_fields(sp, ws, c->stream);
+  // (rows that do not end on 32-byte sectors cross the host link in parts: 16
+  // steps and a read of 97 x 131 x 61, 19 MB, 1,062 us straight, 1,032 through
+  // the planes)
+  bool pinned = !bounce.dev && pageable_access() &&
+                (c->params.nx % 8 == 0 || 6 * bytes <= kDirectRagged);
+  for (int k = 0; k < 6 && pinned; ++k)
+    if (dst[k] && k != 3 && k != 4)  // u's planes are one array
+      pinned = pinned_array(dst[k], k == 2 ? 3 * bytes : bytes);
+  const size_t L = lin_stride(c);
+  hmcsc::FieldsOut out;
+  for (int k = 0; k < 6; ++k)
+    out.p[k] = !dst[k]      ? nullptr
+               : bounce.dev ? reinterpret_cast<float *>(bounce.dev) + (size_t)k * c->N
+               : pinned     ? dst[k]
+                            : c->ws.stage + (size_t)k * L;
+  e = u ? hmcsc::launch_fields(c->sp, c->ws, parity(c), out, c->stream)
+        : hmcsc::launch_density_fields(c->sp, c->ws, out, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "fields kernel");
-  if (!bounce.dev) {
-    const size_t L = lin_stride(c);
+  if (!bounce.dev && !pinned) {
     for (int k = 0; k < 6; ++k) {
       if (!dst[k]) continue;
       e = cudaMemcpyAsync(dst[k], c->ws.stage + (size_t)k * L, bytes,

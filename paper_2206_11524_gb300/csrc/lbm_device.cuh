@@ -959,11 +959,11 @@ __global__ void __launch_bounds__(CollideShape<PARITY, ST, CFG>::threads,
   collide_body<PARITY, ST, PC, S.cs>(p, w, maybe_res, x, y, z);
 }
 
-// Macroscopic fields of the current state into the linear staging planes:
-// rho_1, rho_2, u_macro (Eq. 7) x, y, z, p (Eq. A.6).
+// Macroscopic fields of the current state, linear, x fastest: rho_1, rho_2,
+// u_macro (Eq. 7) x, y, z, p (Eq. A.6), those that `out` has a place for.
 template <int PARITY, int ST, bool PC>
 __global__ void __launch_bounds__(kTile * kFieldsBY * kFieldsBZ)
-    k_fields(StepParams p, Workspace w) {
+    k_fields(StepParams p, Workspace w, FieldsOut out) {
   int x, y, z;
   block_coords<kFieldsBY, kFieldsBZ>(x, y, z);
   const bool maybe_res = block_in_reservoir<kFieldsBY, kFieldsBZ>(p);
@@ -982,23 +982,23 @@ __global__ void __launch_bounds__(kTile * kFieldsBY * kFieldsBZ)
   if (!in_bounds(w.fault, own, p.ntiles * kTile, kFaultGeometry)) own = 0;
   const float fluid = 1.0f - w.ns[own];
   const float fluid2 = PC ? 1.0f - w.ns2[own] : fluid;
-  const long long L = p.nlin;
   const long long n = x + (long long)p.nx * (y + (long long)p.ny * z);
-  if (!in_bounds(w.fault, n, L, kFaultStage)) return;
-  w.stage[n] = r1;
-  w.stage[L + n] = r2;
+  if (!in_bounds(w.fault, n, p.nlin, kFaultStage)) return;
+  if (out.p[0]) out.p[0][n] = r1;
+  if (out.p[1]) out.p[1][n] = r2;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
+    if (!out.p[2 + d]) continue;
     if (PC) {
       const float m = fluid * (j[d].x + 0.5f * r1 * gf[d].x) +
                       fluid2 * (j[d].y + 0.5f * r2 * gf[d].y);
-      w.stage[(2 + d) * L + n] = m / rho;
+      out.p[2 + d][n] = m / rho;
     } else {
       const float m = (j[d].x + 0.5f * r1 * gf[d].x) + (j[d].y + 0.5f * r2 * gf[d].y);
-      w.stage[(2 + d) * L + n] = fluid * m / rho;
+      out.p[2 + d][n] = fluid * m / rho;
     }
   }
-  w.stage[5 * L + n] = (rho + p.G * r1 * r2) * (1.0f / 3.0f);
+  if (out.p[5]) out.p[5][n] = (rho + p.G * r1 * r2) * (1.0f / 3.0f);
 }
 
 // Tiled node index of linear node n = x + nx (y + ny z).

@@ -396,6 +396,12 @@ constexpr unsigned kWaveSpinDefault = 1u << 22;
 // launch may fill (lattices beyond it go to the next set).
 constexpr double kWaveSetL2Share = 0.5;
 
+// Where the fields rho_1, rho_2, u_x, u_y, u_z, p go: device-accessible arrays
+// of N values, NULL for a field that is not wanted.
+struct FieldsOut {
+  float *p[6];
+};
+
 // Per-storage launchers (one translation unit per storage kind).
 #define HMCSC_DECLARE_STORAGE_LAUNCHERS(SUF)                                   \
   cudaError_t launch_density_##SUF(const StepParams &, const Workspace &, int, \
@@ -403,7 +409,7 @@ constexpr double kWaveSetL2Share = 0.5;
   cudaError_t launch_collide_##SUF(const StepParams &, const Workspace &, int, \
                                    int, cudaStream_t);                         \
   cudaError_t launch_fields_##SUF(const StepParams &, const Workspace &, int,  \
-                                  cudaStream_t);                               \
+                                  const FieldsOut &, cudaStream_t);            \
   cudaError_t launch_populations_##SUF(const StepParams &, const Workspace &, int, float *, \
                                        int, int, cudaStream_t);                         \
   cudaError_t launch_init_##SUF(const StepParams &, const Workspace &,         \
@@ -443,7 +449,7 @@ cudaError_t launch_density(const StepParams &p, const Workspace &w, int parity,
 cudaError_t launch_collide_stream(const StepParams &p, const Workspace &w,
                                   int parity, int cfg, cudaStream_t s);
 cudaError_t launch_fields(const StepParams &p, const Workspace &w, int parity,
-                          cudaStream_t s);
+                          const FieldsOut &out, cudaStream_t s);
 // One whole step in a single sweep over the populations (bulk boxes of
 // kSpBY rows x nz / nzc planes, then their seams); needs nx <= kSinglePassMaxNx
 // and 1 <= nzc <= nz.
@@ -475,8 +481,9 @@ cudaError_t launch_resident(const StepParams &p, const Workspace &w, int parity,
 cudaError_t launch_populations(const StepParams &p, const Workspace &w, int parity, float *out,
                                int k0, int nk, cudaStream_t s);
 // The fields that depend on the densities alone (rho_1, rho_2 and p) from
-// w.rho into their planes of w.stage, as k_fields writes them.
-cudaError_t launch_density_fields(const StepParams &p, const Workspace &w, cudaStream_t s);
+// w.rho, as k_fields writes them.
+cudaError_t launch_density_fields(const StepParams &p, const Workspace &w, const FieldsOut &out,
+                                  cudaStream_t s);
 // Observables of w.rho; the kRedK results and the fault word end in *out
 // (device-accessible).
 struct ReduceResult {

@@ -107,17 +107,17 @@ __global__ void k_reduce_final(Workspace w, int blocks, ReduceResult *out) {
   out->value[k] = t;
 }
 
-__global__ void k_density_fields(StepParams p, Workspace w) {
-  const long long N = (long long)p.nx * p.ny * p.nz, L = p.nlin;
+__global__ void k_density_fields(StepParams p, Workspace w, FieldsOut out) {
+  const long long N = (long long)p.nx * p.ny * p.nz;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
     long long tn = tiled_of_linear(p, n);
     if (!in_bounds(w.fault, tn, p.ntiles * kTile, kFaultRhoLoad)) tn = 0;
     const float2 r = w.rho[tn];
     const float r1 = r.x, r2 = r.y, rho = r1 + r2;
-    w.stage[n] = r1;
-    w.stage[L + n] = r2;
-    w.stage[5 * L + n] = (rho + p.G * r1 * r2) * (1.0f / 3.0f);
+    if (out.p[0]) out.p[0][n] = r1;
+    if (out.p[1]) out.p[1][n] = r2;
+    if (out.p[5]) out.p[5][n] = (rho + p.G * r1 * r2) * (1.0f / 3.0f);
   }
 }
 
@@ -209,13 +209,13 @@ cudaError_t launch_collide_stream(const StepParams &p, const Workspace &w,
 }
 
 cudaError_t launch_fields(const StepParams &p, const Workspace &w, int parity,
-                          cudaStream_t s) {
+                          const FieldsOut &out, cudaStream_t s) {
   switch (p.storage) {
-    case kF16: return launch_fields_f16(p, w, parity, s);
-    case kBF16: return launch_fields_bf16(p, w, parity, s);
-    case kF16L: return launch_fields_f16l(p, w, parity, s);
-    case kBF16L: return launch_fields_bf16l(p, w, parity, s);
-    default: return launch_fields_f32(p, w, parity, s);
+    case kF16: return launch_fields_f16(p, w, parity, out, s);
+    case kBF16: return launch_fields_bf16(p, w, parity, out, s);
+    case kF16L: return launch_fields_f16l(p, w, parity, out, s);
+    case kBF16L: return launch_fields_bf16l(p, w, parity, out, s);
+    default: return launch_fields_f32(p, w, parity, out, s);
   }
 }
 
@@ -309,8 +309,9 @@ cudaError_t launch_populations(const StepParams &p, const Workspace &w, int pari
   }
 }
 
-cudaError_t launch_density_fields(const StepParams &p, const Workspace &w, cudaStream_t s) {
-  k_density_fields<<<flat_blocks(p), 256, 0, s>>>(p, w);
+cudaError_t launch_density_fields(const StepParams &p, const Workspace &w, const FieldsOut &out,
+                                  cudaStream_t s) {
+  k_density_fields<<<flat_blocks(p), 256, 0, s>>>(p, w, out);
   return cudaGetLastError();
 }
 

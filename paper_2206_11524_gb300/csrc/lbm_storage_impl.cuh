@@ -111,16 +111,16 @@ cudaError_t HMCSC_NAME(launch_collide)(const StepParams &p, const Workspace &w,
 }
 
 cudaError_t HMCSC_NAME(launch_fields)(const StepParams &p, const Workspace &w,
-                                      int parity, cudaStream_t s) {
+                                      int parity, const FieldsOut &out, cudaStream_t s) {
   const dim3 grid(p.ntx, (p.ny + kFieldsBY - 1) / kFieldsBY,
                   (p.nz + kFieldsBZ - 1) / kFieldsBZ);
   const dim3 block(kTile, kFieldsBY, kFieldsBZ);
   if (w.ns2) {
-    if (parity == 0) k_fields<0, kST, true><<<grid, block, 0, s>>>(p, w);
-    else k_fields<1, kST, true><<<grid, block, 0, s>>>(p, w);
+    if (parity == 0) k_fields<0, kST, true><<<grid, block, 0, s>>>(p, w, out);
+    else k_fields<1, kST, true><<<grid, block, 0, s>>>(p, w, out);
   } else {
-    if (parity == 0) k_fields<0, kST, false><<<grid, block, 0, s>>>(p, w);
-    else k_fields<1, kST, false><<<grid, block, 0, s>>>(p, w);
+    if (parity == 0) k_fields<0, kST, false><<<grid, block, 0, s>>>(p, w, out);
+    else k_fields<1, kST, false><<<grid, block, 0, s>>>(p, w, out);
   }
   return cudaGetLastError();
 }

@@ -100,3 +100,23 @@ def test_two_threads_read_at_once():
     assert not bad
     for g in lats:
         g.close()
+
+
+@pytest.mark.parametrize("shape", [(3, 5, 33), (9, 31, 70), (40, 48, 64)])
+@pytest.mark.parametrize("without", [None, "rho_b", "u", "p"])
+def test_pinned_and_pageable_destinations_agree(shape, without):
+    g, _ = _lattice(shape, "f16l")
+    g.step(3)
+    want = g.fields()
+    n = int(np.prod(shape))
+
+    def pinned(count):            # one value in, so that no array starts on a vector's boundary
+        return torch.empty(count + 1, dtype=torch.float32, pin_memory=True).numpy()[1:]
+
+    out = {k: pinned(n * (3 if k == "u" else 1)) for k in want if k != without}
+    for v in out.values():
+        v[...] = -1.0
+    lbm.lbm_read_fields(g.ctx, out.get("rho_a"), out.get("rho_b"), out.get("u"), out.get("p"))
+    for k, v in out.items():
+        assert np.array_equal(v, want[k].reshape(-1)), k
+    g.close()
