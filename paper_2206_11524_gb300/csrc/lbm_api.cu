@@ -1051,13 +1051,13 @@ void advance_one(lbm_ctx *c) {
 // row-per-warp wavefront step), else one batched density pass and one
 // batched fused pass.
 lbm_status batch_enqueue(lbm_ctx *const *ctxs, int n, int n_steps, cudaStream_t s) {
+  for (int k = 0; k < n; ++k)
+    if (ctxs[k]->fault_seen || (ctxs[k]->fault_host && *(volatile unsigned *)ctxs[k]->fault_host)) {
+      ctxs[k]->fault_seen = true;
+      return fail(ctxs[k], LBM_EINTERNAL,
+                  "a wavefront wait ran out in an earlier step: the state is undefined");
+    }
   if (batch_is_wave(ctxs, n)) {
-    for (int k = 0; k < n; ++k)
-      if (ctxs[k]->fault_seen || (ctxs[k]->fault_host && *(volatile unsigned *)ctxs[k]->fault_host)) {
-        ctxs[k]->fault_seen = true;
-        return fail(ctxs[k], LBM_EINTERNAL,
-                    "a wavefront wait ran out in an earlier step: the state is undefined");
-      }
     static thread_local hmcsc::WaveJob job;
     for (int step = 0; step < n_steps; ++step) {
       job.n = n;

@@ -508,14 +508,17 @@ __host__ __device__ constexpr Shape density_shape(int cfg) {
 // Shapes of the prefetching fused pass (k_collide_pipe): block 32 x by,
 // blocks per SM.  On the 256^3 electrode (us, even / odd step; 168 and 176
 // bytes a node at the copy rate of 6690 GB/s are 421 and 441): half offsets
-// 559/633 in shape 6, 438/528 in shapes 9/8; local half offsets 697/868 in
-// shape 6, 471/564 in shape 9, and 551 on even steps without its streaming
-// stores; float32 (320 bytes: 803) 774/902 in shape 6, 816/891 in shape 7,
-// 778/983 in shape 9.  Even steps are bound by HBM.  Odd ones store rows
-// shifted by a node, which leave part of a sector at either end, and keep 18
-// addresses: the local storages take 168 registers there.  Staging the
-// stencil pays for the 16-bit storages, whose bytes are fewer than their
-// stencil's loads can hide behind; float32 is bound by its bytes either way.
+// 519/586 in shape 6, 430/520 in shapes 9/8 (scalar code, 8-byte copies and
+// no stencil ring on even steps: 606/737); local half offsets 693/728 in
+// shape 6, 455/553 in shape 9 (726/810), and 547 on even steps without its
+// streaming stores; float32 (320 bytes: 803) 774/885 in shape 6, 816/881 in
+// shape 7 (837/967), 778/985 in shape 9.  Even steps are bound by HBM.  Odd
+// ones store rows shifted by a node, which leave part of a sector at either
+// end, and keep 18 addresses: they issue 753-788 instructions a node, 61 % of
+// the slots, and the local storages take 168 registers.  Staging the stencil
+// pays for the 16-bit storages, whose bytes are fewer than their stencil's
+// loads can hide behind; float32 is bound by its bytes either way.  More
+// blocks per SM spill: at 10 and 9, half offsets run 525/705.
 struct PipeCfg {
   int by, minb_even, minb_odd, minb_even_local, minb_odd_local;
   bool ring;  // neighbour densities and adhesion sources also staged in
@@ -1081,6 +1084,12 @@ __global__ void k_init_equilibrium(StepParams p, Workspace w,
 // stays race-free: the collision of node n touches only the slots holding
 // n's own populations, whose density part has finished reading them before
 // n's flag is set.
+// One float32 step of 256^3 takes 1,103 us (1,156 with scalar arithmetic and
+// rows not uniform) and moves 335 bytes a node, against 1,210 us and 476 in
+// two passes.  What bounds it is the chain of each item -- copies from DRAM,
+// flags, stencil from L2 -- at 16 warps per SM: fewer instructions (divisions
+// as multiplications, copies in chunks) did not shorten it, nor did
+// publishing before the collision's stores.
 struct WaveCfg {
   int by, minb, minb_local;
 };

@@ -52,9 +52,9 @@ constexpr float kHalfScale = 16384.0f, kHalfUnscale = 1.0f / 16384.0f;
 // Packed arithmetic on the pair (sigma = 1, 2): one instruction does both
 // components, each rounded as the scalar operation would be (add.f32x2,
 // mul.f32x2, fma.f32x2).  Both components take the same steps everywhere on
-// the path, and the 16-bit fused passes are bound by instruction issue
-// (1,115-1,289 instructions a node in scalar form), so the pairs stay pairs
-// from the load to the store.  A subtraction is a fused multiply-add with
+// the path, and the 16-bit fused passes were bound by instruction issue
+// (1,115-1,289 instructions a node in scalar form, 691-788 now, row copies
+// included), so the pairs stay pairs from the load to the store.  A subtraction is a fused multiply-add with
 // -1, which rounds once like the subtraction it stands for.
 // A packed product that feeds a packed sum is fused with it by the assembler
 // (measured: mul2 into add2 rounds once, .rn or not), so where both roundings

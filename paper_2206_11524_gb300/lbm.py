@@ -449,13 +449,14 @@ class Lattice:
 
     def set_wavefront(self, shape, lag=0):
         """Wavefront lbm_step of tile shape `shape` (1: 32 x 4, 2: 32 x 2,
-        3: 32 x 8 nodes; 0: off) with densities `lag` planes ahead (0:
-        default); lbm_batch_step then also steps such lattices together in
+        3: 32 x 8 nodes; 0: lbm_step's own choice) with densities `lag`
+        planes ahead (0: default); lbm_batch_step then also steps such lattices together in
         one wavefront launch."""
         lbm_set_wavefront(self.ctx, shape, lag)
 
     def wavefront(self):
-        """(shape, lag) of the wavefront step in use (shape 0: off)."""
+        """(shape, lag) of the wavefront step asked for (shape 0: none, the
+        step is lbm_step's own choice)."""
         return lbm_get_wavefront(self.ctx)
 
     def set_launch_config(self, density_cfg=0, even_cfg=0, odd_cfg=0):
