@@ -321,10 +321,13 @@ bool pageable_access() {
   });
   return yes[dev];
 }
-// Is the array pinned from its first byte to its last, at its host address?
-// (Kernel writes reach pinned memory at the copy engine's 193 GB/s, and the
-// six copies of small fields cost 2.5 us each.)
+// May a kernel write floats to the array: is it pinned from its first byte to
+// its last, at its host address, and does it start where a float may?  (A copy
+// takes any address; a kernel's store at half a float faults.  Kernel writes
+// reach pinned memory at the copy engine's 193 GB/s, and the six copies of
+// small fields cost 2.5 us each.)
 bool pinned_array(const void *p, size_t bytes) {
+  if ((uintptr_t)p % sizeof(float) != 0) return false;
   const char *end[2] = {(const char *)p, (const char *)p + bytes - 1};
   for (const char *q : end) {
     cudaPointerAttributes at;
