@@ -8,6 +8,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <initializer_list>
 #include <mutex>
 #include <string>
 #include <thread>
@@ -126,14 +127,29 @@ bool fault_slot_take(HostSlot **host, HostSlot **dev, int *slot) {
   return true;
 }
 
-// The read-back buffer, for a call that needs `bytes` of it: host and device
-// views, or NULL when there is none, it is too small or another thread has it.
+// Is the address one that only the device may write?  (A copy there is the
+// runtime's to refuse; a store of the host's would end the process.)
+bool device_only(const void *p) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) == cudaSuccess) return at.type == cudaMemoryTypeDevice;
+  cudaGetLastError();
+  return false;
+}
+
+// The read-back buffer, for a call that needs `bytes` of it to fill the arrays
+// dst (NULL: not wanted): host and device views, or NULL when there is none, it
+// is too small, another thread has it or the host cannot write one of the
+// arrays.
 struct Bounce {
   std::unique_lock<std::mutex> lock;
   char *host = nullptr;
   char *dev = nullptr;
-  Bounce(size_t bytes, size_t most) : lock(g_bounce_mu, std::defer_lock) {
-    if (!g_fault_host || bytes > most || !lock.try_lock()) return;
+  Bounce(size_t bytes, size_t most, std::initializer_list<float *> dst)
+      : lock(g_bounce_mu, std::defer_lock) {
+    if (!g_fault_host || bytes > most) return;
+    for (const float *p : dst)
+      if (p && device_only(p)) return;
+    if (!lock.try_lock()) return;
     host = reinterpret_cast<char *>(g_fault_host + kFaultSlots);
     dev = reinterpret_cast<char *>(g_fault_dev + kFaultSlots);
   }
@@ -616,7 +632,7 @@ lbm_status lbm_get_populations(lbm_ctx *c, float *f) {
   // into the staging planes, as many of the 38 at a time as fit
   const size_t plane = sizeof(float) * (size_t)c->N;
   bool synced;
-  Bounce bounce(2 * kQ * plane, kBounceBytes);
+  Bounce bounce(2 * kQ * plane, kBounceBytes, {f});
   if (bounce.dev) {
     cudaError_t e = hmcsc::launch_populations(c->sp, c->ws, parity(c),
                                               reinterpret_cast<float *>(bounce.dev), 0, 2 * kQ,
@@ -812,7 +828,7 @@ lbm_status lbm_read_fields(lbm_ctx *c, float *rho_a, float *rho_b, float *u,
   // small fields are written into the read-back buffer, fields for pinned
   // arrays straight into those, others into the staging planes, from which
   // they are copied; without u the densities say all
-  Bounce bounce(6 * bytes, kBounceFields);
+  Bounce bounce(6 * bytes, kBounceFields, {rho_a, rho_b, u, p});
   // (rows that do not end on 32-byte sectors cross the host link in parts: 16
   // steps and a read of 97 x 131 x 61, 19 MB, 1,062 us straight, 1,032 through
   // the planes)

@@ -6,6 +6,8 @@
 #include <cstdio>
 #include <cstring>
 
+#include <sys/mman.h>
+
 #include "api_fakes.h"
 #include "lbm.h"
 #include "lbm_internal.cuh"
@@ -125,7 +127,7 @@ struct Lattice {
 // A pinned destination that does not start on a float gets its fields through
 // the staging planes: a kernel cannot store floats there.
 static void misaligned_destination() {
-  for (const int nx : {16, 64}) {            // through the buffer, and too large for it
+  for (const int nx : {8, 64}) {            // through the buffer, and too large for it
     Lattice l(nx, 32, 16);
     std::vector<char> mem(5 * 4 * l.N + 64);
     ranges = {{mem.data(), mem.size(), cudaMemoryTypeHost, 0}};
@@ -149,9 +151,34 @@ static void misaligned_destination() {
   }
 }
 
+// An address the host cannot write is refused by the copy to it, whatever the
+// lattice's size; the host never writes there itself.
+static void device_destination() {
+  for (const int nx : {8, 64}) {
+    Lattice l(nx, 32, 16);
+    const size_t bytes = 4 * 38 * l.N;
+    float *at = (float *)mmap(nullptr, bytes, PROT_NONE, MAP_PRIVATE | MAP_ANONYMOUS, -1, 0);
+    CHECK(at != MAP_FAILED);
+    ranges = {{(const char *)at, bytes, cudaMemoryTypeDevice, 0}};
+    std::vector<float> host(38 * l.N);
+    CHECK(lbm_read_fields(l.ctx, at, nullptr, nullptr, nullptr) == LBM_ECUDA);
+    CHECK(lbm_read_fields(l.ctx, nullptr, at, nullptr, nullptr) == LBM_ECUDA);
+    CHECK(lbm_read_fields(l.ctx, host.data(), nullptr, at, nullptr) == LBM_ECUDA);
+    CHECK(lbm_read_fields(l.ctx, nullptr, nullptr, nullptr, at) == LBM_ECUDA);
+    CHECK(lbm_get_populations(l.ctx, at) == LBM_ECUDA);
+    CHECK(lbm_read_fields(l.ctx, host.data(), nullptr, nullptr, host.data() + l.N) == LBM_OK);
+    CHECK(host[l.N - 1] == l.N - 1 && host[l.N] == 5000.0f);
+    CHECK(lbm_get_populations(l.ctx, host.data()) == LBM_OK);
+    CHECK(host[37 * l.N] == 37000.0f);
+    ranges.clear();
+    munmap(at, bytes);
+  }
+}
+
 int main(int argc, char **argv) {
   const std::string name = argc > 1 ? argv[1] : "";
   if (name == "misaligned_destination") misaligned_destination();
+  else if (name == "device_destination") device_destination();
   else return std::printf("no check '%s'\n", name.c_str()), 2;
   if (failures == 0) std::printf("ok\n");
   return failures != 0;

@@ -1,6 +1,8 @@
 """Host arrays that lbm_read_fields and lbm_get_populations are handed: where
 they lie and how they are aligned decides how the results travel, never what
 they are."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -49,4 +51,22 @@ def test_pinned_arrays_at_any_byte(shape, offset):
     lbm.lbm_read_fields(g.ctx, out["rho_a"], out["rho_b"], out["u"], out["p"])
     for k, v in out.items():
         assert np.array_equal(v, want[k].reshape(-1)), k
+    g.close()
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_device_addresses_are_the_runtimes_to_refuse(shape):
+    """The copy to the array decides, as for a large lattice: it is refused, or
+    made; the process lives and so does the lattice."""
+    g = _lattice(shape)
+    want = g.fields()["rho_a"].reshape(-1)
+    d = torch.zeros(38 * want.size, dtype=torch.float32, device="cuda")
+    torch.cuda.synchronize()
+    at = ctypes.cast(d.data_ptr(), ctypes.POINTER(ctypes.c_float))
+    st = lbm.load().lbm_read_fields(g.ctx, at, None, None, None)
+    assert st in (lbm.LBM_OK, lbm.LBM_ECUDA)
+    if st == lbm.LBM_OK:
+        assert np.array_equal(d[:want.size].cpu().numpy(), want)
+    assert lbm.load().lbm_get_populations(g.ctx, at) == st
+    assert np.array_equal(g.fields()["rho_a"].reshape(-1), want)
     g.close()
