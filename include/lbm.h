@@ -175,7 +175,9 @@ LBM_API lbm_status lbm_set_bc_velocity(lbm_ctx *ctx, int face, int layers,
  * shapes of the caller's (lbm_set_launch_config) takes up to 256 steps per
  * launch instead, and a larger float32 lattice whose planes in flight stay in
  * L2 takes the wavefront launch with a lag of the library's choice, with the
- * same results bit for bit; all waits are bounded like the wavefront's.  n_steps = 0 is a no-op.  EINTERNAL (and
+ * same results bit for bit; all waits are bounded like the wavefront's, and
+ * where such a launch is refused (a stream that may use only some of the SMs)
+ * the two passes run instead.  n_steps = 0 is a no-op.  EINTERNAL (and
  * nothing enqueued) when a device fault was reported for the current state:
  * by a synchronising call (below), or by a launch that already ran, through
  * a host-mapped word the kernel sets (no stream wait). */

@@ -45,6 +45,7 @@ struct lbm_ctx {
   bool launch_cfg_set;    // by the caller: lbm_step keeps the passes they are for
   int auto_lag;           // wave_auto_lag: > 0: lbm_step's own choice is the
                           // wavefront launch with this lag
+  bool choice_refused;    // lbm_step's own choice could not be launched
   int single_pass_zc;     // > 0: lbm_step sweeps once, boxes of this many planes
   int wave_cfg;           // > 0: lbm_step is one wavefront launch of this shape
   int wave_lag;           // planes between a plane's density and its collision
@@ -450,6 +451,7 @@ lbm_status lbm_create(const lbm_params *params, void *d_workspace,
   c->launch_cfg[2] = f32 ? 7 : local ? 9 : 8;
   c->launch_cfg_set = false;
   c->auto_lag = hmcsc::wave_auto_lag(sp);
+  c->choice_refused = false;
   c->single_pass_zc = 0;
   c->wave_cfg = 0;
   c->wave_lag = hmcsc::kWaveLagDefault;
@@ -723,35 +725,45 @@ lbm_status lbm_step(lbm_ctx *c, int n_steps) {
                 "load a checkpoint or set a new state");
   }
   for (int k = 0; k < n_steps; ++k) {
-    // small lattices stay on the device for several steps; a reservoir change
+    // A lattice whose caller asked for no step in particular takes the launch
+    // that suits its size.  Such a launch wants the whole device (a cluster of
+    // 16 blocks, or all blocks resident at once), which a stream limited to
+    // some of the SMs refuses; nothing has been enqueued then, and the two
+    // passes, which run anywhere, take over for good.
+    const bool own_choice = c->wave_cfg == 0 && c->single_pass_zc == 0 && !c->launch_cfg_set &&
+                            !c->choice_refused;
+    // Small lattices stay on the device for several steps; a reservoir change
     // takes effect at the end of a step, so the step it was made for is taken
-    // on its own
-    if (c->wave_cfg == 0 && c->single_pass_zc == 0 && !c->launch_cfg_set &&
-        c->sp.ntiles <= hmcsc::kResidentTiles &&
+    // on its own.
+    if (own_choice && c->sp.ntiles <= hmcsc::kResidentTiles &&
         memcmp(&c->sp.res, &c->res_current, sizeof(hmcsc::Reservoirs)) == 0) {
       const int m = n_steps - k < hmcsc::kResidentSteps ? n_steps - k : hmcsc::kResidentSteps;
       cudaError_t e = hmcsc::launch_resident(c->sp, c->ws, parity(c), m, c->wave_spin,
                                              c->wave_hold >= 0, c->stream);
-      if (e != cudaSuccess) return cuda_fail(c, e, "resident kernel");
-      for (int q = 0; q < m; ++q) {
+      if (e == cudaSuccess) {
+        for (int q = 0; q < m; ++q) {
+          c->rho_at = c->t;
+          finish_step(c);
+        }
+        k += m - 1;
+        continue;
+      }
+      cudaGetLastError();  // (an error of the context itself meets the passes too)
+      c->choice_refused = true;
+    }
+    if (c->wave_cfg > 0 || (own_choice && c->auto_lag > 0 && !c->choice_refused)) {
+      const bool asked = c->wave_cfg > 0;
+      cudaError_t e = hmcsc::launch_wave(c->sp, c->ws, parity(c), asked ? c->wave_cfg : 2,
+                                         asked ? c->wave_lag : c->auto_lag, c->wave_spin,
+                                         c->wave_hold, c->stream);
+      if (e == cudaSuccess) {
         c->rho_at = c->t;
         finish_step(c);
+        continue;
       }
-      k += m - 1;
-      continue;
-    }
-    // the wavefront launch, asked for or chosen (for a lattice whose caller
-    // asked for no step in particular)
-    const bool own_choice =
-        c->wave_cfg == 0 && c->single_pass_zc == 0 && !c->launch_cfg_set && c->auto_lag > 0;
-    if (c->wave_cfg > 0 || own_choice) {
-      cudaError_t e = hmcsc::launch_wave(c->sp, c->ws, parity(c), own_choice ? 2 : c->wave_cfg,
-                                         own_choice ? c->auto_lag : c->wave_lag, c->wave_spin,
-                                         c->wave_hold, c->stream);
-      if (e != cudaSuccess) return cuda_fail(c, e, "wavefront kernel");
-      c->rho_at = c->t;
-      finish_step(c);
-      continue;
+      if (asked) return cuda_fail(c, e, "wavefront kernel");
+      cudaGetLastError();
+      c->choice_refused = true;
     }
     if (c->single_pass_zc > 0) {
       // runs of about single_pass_zc planes along z

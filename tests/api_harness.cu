@@ -175,10 +175,40 @@ static void device_destination() {
   }
 }
 
+// Where the launch lbm_step chose by itself is refused, the steps run as two
+// passes, from then on without asking again; a step the caller asked for
+// reports the error.
+static void refused_choice() {
+  const struct { int nx, ny, nz; const char *name; } own[] = {{32, 32, 32, "resident"}, {128, 128, 128, "wave"}};
+  for (const auto &o : own)
+    for (const cudaError_t e : {cudaErrorCooperativeLaunchTooLarge, cudaErrorLaunchOutOfResources}) {
+      Lattice l(o.nx, o.ny, o.nz);
+      CHECK(lbm_step(l.ctx, 1) == LBM_OK);
+      CHECK(launched[o.name] == 1 && launched["density"] == 0);
+      refused = {{o.name, e}};
+      CHECK(lbm_step(l.ctx, 3) == LBM_OK);
+      CHECK(cudaGetLastError() == cudaSuccess);
+      CHECK(launched["density"] == 3 && launched["collide"] == 3);
+      CHECK(lbm_time(l.ctx) == 4);
+      refused.clear();
+      CHECK(lbm_step(l.ctx, 2) == LBM_OK);
+      CHECK(launched["density"] == 5 && launched[o.name] == 1);
+    }
+  Lattice l(32, 32, 32);
+  CHECK(lbm_set_wavefront(l.ctx, 2, 4) == LBM_OK);
+  refused = {{"wave", cudaErrorCooperativeLaunchTooLarge}};
+  CHECK(lbm_step(l.ctx, 1) == LBM_ECUDA);
+  refused = {{"density", cudaErrorIllegalAddress}, {"resident", cudaErrorIllegalAddress}};
+  Lattice m(32, 32, 32);
+  CHECK(lbm_step(m.ctx, 1) == LBM_ECUDA);  // an error of the context stays one
+  refused.clear();
+}
+
 int main(int argc, char **argv) {
   const std::string name = argc > 1 ? argv[1] : "";
   if (name == "misaligned_destination") misaligned_destination();
   else if (name == "device_destination") device_destination();
+  else if (name == "refused_choice") refused_choice();
   else return std::printf("no check '%s'\n", name.c_str()), 2;
   if (failures == 0) std::printf("ok\n");
   return failures != 0;
