@@ -235,7 +235,7 @@ LBM_API lbm_status lbm_get_wavefront(const lbm_ctx *ctx, int *shape, int *lag);
  * lbm_density (rho_sigma of Eq. A.4 at every node) followed by
  * lbm_collide_stream (Eqs. 3-6, A.3, 1 and the reservoirs) is exactly one
  * lbm_step(ctx, 1).  lbm_collide_stream without a preceding lbm_density at
- * the same time step is ESTATE. */
+ * the same time step is ESTATE; EINTERNAL as for lbm_step. */
 LBM_API lbm_status lbm_density(lbm_ctx *ctx);
 LBM_API lbm_status lbm_collide_stream(lbm_ctx *ctx);
 
@@ -322,7 +322,8 @@ LBM_API lbm_status lbm_batch_step(lbm_ctx *const *ctxs, int n, int n_steps,
  * runs those steps and advances every context's host state; it is valid as
  * long as each context still has the time parity, density buffers and
  * reservoirs it had at capture (after an even number of steps they return),
- * else the launch returns ESTATE and nothing runs.  Reservoir changes must
+ * else the launch returns ESTATE and nothing runs, as it returns EINTERNAL for
+ * a context whose state a wait left undefined.  Reservoir changes must
  * have taken effect (one step after lbm_set_bc) before capture.  The graph
  * refers to the contexts: destroy it before them. */
 typedef struct lbm_graph lbm_graph;

@@ -272,6 +272,17 @@ lbm_status judge_fault(lbm_ctx *c, unsigned v) {
               "the bounds-checked build recorded an out-of-range access (fault word 0x%x)", v);
 }
 
+// Has a wait of an earlier launch run out?  Then EINTERNAL: no call advances
+// the state until it is replaced.  (No wait for the stream: what the host-mapped
+// word says so far.)
+lbm_status refuse_undefined(lbm_ctx *c) {
+  if (!c->fault_seen && !(c->fault_host && *(volatile unsigned *)c->fault_host)) return LBM_OK;
+  c->fault_seen = true;
+  return fail(c, LBM_EINTERNAL,
+              "a wavefront wait ran out in an earlier step: the state is undefined; "
+              "load a checkpoint or set a new state");
+}
+
 // Wait for the stream, then judge the fault word: one wait for both where the
 // word can be copied to the context's slot.  *synced: the stream has drained
 // (results copied before are there even when a fault is reported).
@@ -695,6 +706,7 @@ lbm_status lbm_density(lbm_ctx *c) {
   if (!c) return LBM_EINVAL;
   if (!c->have_geometry || !c->have_state)
     return fail(c, LBM_ESTATE, "set geometry and state before stepping");
+  if (const lbm_status st = refuse_undefined(c)) return st;
   cudaError_t e = hmcsc::launch_density(c->sp, c->ws, parity(c), c->launch_cfg[0], c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "density kernel");
   c->rho_at = c->t;
@@ -705,6 +717,7 @@ lbm_status lbm_collide_stream(lbm_ctx *c) {
   if (!c) return LBM_EINVAL;
   if (c->rho_at != c->t)
     return fail(c, LBM_ESTATE, "lbm_density must precede lbm_collide_stream");
+  if (const lbm_status st = refuse_undefined(c)) return st;
   cudaError_t e = hmcsc::launch_collide_stream(c->sp, c->ws, parity(c),
                                                 c->launch_cfg[1 + parity(c)], c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "collide/stream kernel");
@@ -718,12 +731,7 @@ lbm_status lbm_step(lbm_ctx *c, int n_steps) {
   if (n_steps == 0) return LBM_OK;
   if (!c->have_geometry || !c->have_state)
     return fail(c, LBM_ESTATE, "set geometry and state before stepping");
-  if (c->fault_seen || (c->fault_host && *(volatile unsigned *)c->fault_host)) {
-    c->fault_seen = true;
-    return fail(c, LBM_EINTERNAL,
-                "a wavefront wait ran out in an earlier step: the state is undefined; "
-                "load a checkpoint or set a new state");
-  }
+  if (const lbm_status st = refuse_undefined(c)) return st;
   for (int k = 0; k < n_steps; ++k) {
     // A lattice whose caller asked for no step in particular takes the launch
     // that suits its size.  Such a launch wants the whole device (a cluster of
@@ -1083,11 +1091,7 @@ void advance_one(lbm_ctx *c) {
 // batched fused pass.
 lbm_status batch_enqueue(lbm_ctx *const *ctxs, int n, int n_steps, cudaStream_t s) {
   for (int k = 0; k < n; ++k)
-    if (ctxs[k]->fault_seen || (ctxs[k]->fault_host && *(volatile unsigned *)ctxs[k]->fault_host)) {
-      ctxs[k]->fault_seen = true;
-      return fail(ctxs[k], LBM_EINTERNAL,
-                  "a wavefront wait ran out in an earlier step: the state is undefined");
-    }
+    if (const lbm_status st = refuse_undefined(ctxs[k])) return st;
   if (batch_is_wave(ctxs, n)) {
     static thread_local hmcsc::WaveJob job;
     for (int step = 0; step < n_steps; ++step) {
@@ -1217,6 +1221,7 @@ lbm_status lbm_batch_graph_launch(lbm_graph *g, void *cuda_stream) {
         c->bc_version != g->bc0[k] ||
         memcmp(&c->sp.res, &c->res_current, sizeof(hmcsc::Reservoirs)) != 0)
       return fail(c, LBM_ESTATE, "lattice changed since the graph was captured");
+    if (const lbm_status st = refuse_undefined(c)) return st;
   }
   cudaError_t e = cudaGraphLaunch(g->exec, (cudaStream_t)cuda_stream);
   if (e != cudaSuccess) return cuda_fail(g->ctxs[0], e, "graph launch");

@@ -24,6 +24,7 @@ static int failures = 0;
 // ---- launchers ----
 
 static hmcsc::FieldsOut last_fields;
+static unsigned *last_fault_host;  // of the workspace density was last launched on
 
 namespace hmcsc {
 size_t workspace_bytes(long long nx, long long ny, long long nz, int, bool pc, Workspace *w, char *b) {
@@ -49,7 +50,8 @@ cudaError_t launch_init_equilibrium(const StepParams &, const Workspace &, const
                                     cudaStream_t) { return launch("init"); }
 cudaError_t launch_geometry(const StepParams &, const Workspace &, const float *, const float *, const float *,
                             cudaStream_t) { return launch("geometry"); }
-cudaError_t launch_density(const StepParams &, const Workspace &, int, int, cudaStream_t) {
+cudaError_t launch_density(const StepParams &, const Workspace &w, int, int, cudaStream_t) {
+  last_fault_host = w.fault_host;
   return launch("density");
 }
 cudaError_t launch_collide_stream(const StepParams &, const Workspace &, int, int, cudaStream_t) {
@@ -204,11 +206,38 @@ static void refused_choice() {
   refused.clear();
 }
 
+// After a wait that ran out no call advances the state, until a new one is set.
+static void undefined_state() {
+  Lattice l(32, 32, 32), other(32, 32, 32);
+  lbm_ctx *both[2] = {other.ctx, l.ctx};
+  lbm_graph *g = nullptr;
+  CHECK(lbm_batch_graph_create(both, 2, 2, (void *)1, &g) == LBM_OK);
+  CHECK(lbm_batch_graph_launch(g, (void *)1) == LBM_OK);
+  CHECK(lbm_density(l.ctx) == LBM_OK);
+  *last_fault_host = LBM_FAULT_WAIT;
+  launched.clear();
+  CHECK(lbm_step(l.ctx, 1) == LBM_EINTERNAL);
+  CHECK(lbm_collide_stream(l.ctx) == LBM_EINTERNAL);
+  CHECK(lbm_density(l.ctx) == LBM_EINTERNAL);
+  CHECK(lbm_batch_step(both, 2, 2, (void *)1) == LBM_EINTERNAL);
+  CHECK(lbm_batch_graph_launch(g, (void *)1) == LBM_EINTERNAL);
+  CHECK(launched.empty());
+  CHECK(lbm_time(l.ctx) == 2 && lbm_time(other.ctx) == 2);
+  CHECK(strlen(lbm_last_error(l.ctx)) > 0);
+  const std::vector<float> one(l.N, 1.0f);
+  for (lbm_ctx *c : both) CHECK(lbm_init_equilibrium(c, one.data(), one.data()) == LBM_OK);
+  CHECK(lbm_batch_graph_launch(g, (void *)1) == LBM_OK);
+  CHECK(lbm_density(l.ctx) == LBM_OK && lbm_collide_stream(l.ctx) == LBM_OK);
+  CHECK(lbm_time(l.ctx) == 3);
+  lbm_batch_graph_destroy(g);
+}
+
 int main(int argc, char **argv) {
   const std::string name = argc > 1 ? argv[1] : "";
   if (name == "misaligned_destination") misaligned_destination();
   else if (name == "device_destination") device_destination();
   else if (name == "refused_choice") refused_choice();
+  else if (name == "undefined_state") undefined_state();
   else return std::printf("no check '%s'\n", name.c_str()), 2;
   if (failures == 0) std::printf("ok\n");
   return failures != 0;

@@ -30,7 +30,8 @@ def harness(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("check", ["misaligned_destination", "device_destination", "refused_choice"])
+@pytest.mark.parametrize("check", ["misaligned_destination", "device_destination", "refused_choice",
+                                   "undefined_state"])
 def test_host_side(harness, check):
     out = subprocess.run([harness, check], capture_output=True, text=True)
     assert out.returncode == 0 and out.stdout.strip() == "ok", out.stdout + out.stderr
