@@ -170,12 +170,13 @@ LBM_API lbm_status lbm_set_bc_velocity(lbm_ctx *ctx, int face, int layers,
  * the context's stream.  Each step launches the density pass and the fused
  * force/collide/bounce-back/stream pass, or the single-pass sweep when
  * lbm_set_single_pass enabled it, or the wavefront launch when
- * lbm_set_wavefront enabled it.  A small lattice (up to 4,608 x-tiles: nx /
- * 32, rounded up, times ny nz) without those two settings and without launch
- * shapes of the caller's (lbm_set_launch_config) takes up to 256 steps per
- * launch instead, and a larger float32 lattice whose planes in flight stay in
- * L2 takes the wavefront launch with a lag of the library's choice, with the
- * same results bit for bit; all waits are bounded like the wavefront's, and
+ * lbm_set_wavefront enabled it.  A context whose caller used none of
+ * lbm_set_single_pass, lbm_set_wavefront and lbm_set_launch_config, or
+ * lbm_set_automatic_step since, takes the step that suits its size, with the
+ * same results bit for bit: a small lattice (up to 4,608 x-tiles: nx / 32,
+ * rounded up, times ny nz) up to 256 steps per launch, a larger float32 lattice
+ * whose planes in flight stay in L2 the wavefront launch with a lag of the
+ * library's choice; all waits are bounded like the wavefront's, and
  * where such a launch is refused (a stream that may use only some of the SMs)
  * the two passes run instead.  n_steps = 0 is a no-op.  EINTERNAL (and
  * nothing enqueued) when a device fault was reported for the current state:
@@ -183,8 +184,12 @@ LBM_API lbm_status lbm_set_bc_velocity(lbm_ctx *ctx, int face, int layers,
  * a host-mapped word the kernel sets (no stream wait). */
 LBM_API lbm_status lbm_step(lbm_ctx *ctx, int n_steps);
 
-/* Single-pass stepping for lbm_step (planes > 0; 0 = two passes, the
- * default): each step reads every population once.  The lattice is cut into
+/* Back to the step of the library's choice (lbm_step), as in a new context:
+ * undoes lbm_set_single_pass, lbm_set_wavefront and lbm_set_launch_config.
+ * EINVAL: NULL ctx. */
+LBM_API lbm_status lbm_set_automatic_step(lbm_ctx *ctx);
+
+/* Single-pass stepping for lbm_step (planes > 0; 0 = two passes): each step reads every population once.  The lattice is cut into
  * boxes of full x-rows, 8 rows by `planes` planes; one launch marches every
  * box along z, computing the densities of the next plane into shared memory
  * and colliding the current plane's inner rows with them; the last row and
@@ -194,9 +199,9 @@ LBM_API lbm_status lbm_step(lbm_ctx *ctx, int n_steps);
  * lbm_collide_stream and the batched entry points keep the two passes. */
 LBM_API lbm_status lbm_set_single_pass(lbm_ctx *ctx, int planes);
 
-/* Wavefront stepping for lbm_step (shape > 0; 0, the default, leaves the step
- * to lbm_step; it takes precedence over lbm_set_single_pass): each step is one persistent
- * cooperative launch over work items, a tile of 32 x by nodes of one plane
+/* Wavefront stepping for lbm_step (shape > 0; 0 = two passes, or the single
+ * pass if that is set; shapes take precedence over it): each step is one
+ * persistent cooperative launch over work items, a tile of 32 x by nodes of one plane
  * each (shape 1: by = 4, 2: by = 2, 3: by = 8), taken in plane order from an
  * atomic ticket.  An item sums the populations of one plane's tile into the
  * density array and collides and streams the tile `lag` planes behind it
@@ -227,7 +232,7 @@ LBM_API lbm_status lbm_set_wavefront(lbm_ctx *ctx, int shape, int lag);
  * completing.  EINVAL if the index is outside the flag words. */
 LBM_API lbm_status lbm_set_wavefront_limits(lbm_ctx *ctx, uint32_t spin_limit,
                                             int64_t withhold_flag);
-/* The wavefront shape (0: off) and lag in use, to *shape and *lag (either
+/* The wavefront shape asked for (0: none) and its lag, to *shape and *lag (either
  * may be NULL).  Errors: EINVAL (NULL ctx). */
 LBM_API lbm_status lbm_get_wavefront(const lbm_ctx *ctx, int *shape, int *lag);
 
@@ -287,7 +292,8 @@ LBM_API const char *lbm_last_error(const lbm_ctx *ctx);
  * storage on a 256^3 lattice (float32 1/6/7, half and bfloat16 offsets 0/9/8,
  * local offsets 0/9/9).  Results do not depend on the choice; speed does (the
  * autotuner measures them per lattice size and storage).  Once they are set,
- * lbm_step runs the two passes in them, small lattices included.  EINVAL if
+ * lbm_step runs the two passes in them, small lattices included, until
+ * lbm_set_automatic_step.  EINVAL if
  * out of range. */
 #define LBM_DENSITY_CONFIGS 3
 #define LBM_COLLIDE_CONFIGS 10

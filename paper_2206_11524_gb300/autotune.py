@@ -211,8 +211,9 @@ def apply(lattice, table: TuneTable | None = None, tune_if_missing=True,
                             wavefront=wavefront)
         table.put(nx, ny, nz, storage, cfg, timings)
     if cfg is not None:
+        lattice.set_automatic_step()
         if cfg[0] >= 0:
             lbm.lbm_set_launch_config(lattice.ctx, *cfg[:3])
-        lattice.set_single_pass(cfg[3] if len(cfg) > 3 else 0)
-        lattice.set_wavefront(*(cfg[4:6] if len(cfg) > 5 else (0, 0)))
+            lattice.set_single_pass(cfg[3] if len(cfg) > 3 else 0)
+            lattice.set_wavefront(*(cfg[4:6] if len(cfg) > 5 else (0, 0)))
     return cfg

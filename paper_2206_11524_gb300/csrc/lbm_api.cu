@@ -42,7 +42,7 @@ struct lbm_ctx {
   bool have_state;
   uint64_t bc_version;    // bumped by every lbm_set_bc
   int launch_cfg[3];      // launch shapes: density, even fused, odd fused
-  bool launch_cfg_set;    // by the caller: lbm_step keeps the passes they are for
+  bool step_set;          // the caller asked for a step: lbm_step chooses none
   int auto_lag;           // wave_auto_lag: > 0: lbm_step's own choice is the
                           // wavefront launch with this lag
   bool choice_refused;    // lbm_step's own choice could not be launched
@@ -376,6 +376,21 @@ lbm_status upload(lbm_ctx *c, float *dst, const float *src, size_t n) {
   return LBM_OK;
 }
 
+// No step asked for, and the launch shapes measured fastest for the storage on
+// the 256^3 electrode (the tuner refines them per size).
+void automatic_step(lbm_ctx *c) {
+  const bool local = hmcsc::storage_local(c->sp.storage);
+  const bool f32 = c->sp.storage == hmcsc::kF32;
+  c->launch_cfg[0] = f32 ? 1 : 0;
+  c->launch_cfg[1] = f32 ? 6 : 9;
+  c->launch_cfg[2] = f32 ? 7 : local ? 9 : 8;
+  c->step_set = false;
+  c->choice_refused = false;
+  c->single_pass_zc = 0;
+  c->wave_cfg = 0;
+  c->wave_lag = hmcsc::kWaveLagDefault;
+}
+
 // Host bookkeeping after the fused pass of a step.
 void finish_step(lbm_ctx *c) {
   // The reservoirs in force now reset their layers at the end of this step.
@@ -453,19 +468,8 @@ lbm_status lbm_create(const lbm_params *params, void *d_workspace,
   c->have_geometry = false;
   c->have_state = false;
   c->bc_version = 0;
-  // start from the shapes measured fastest for the storage on the 256^3
-  // electrode (the tuner refines them per size)
-  const bool local = hmcsc::storage_local(params->storage);
-  const bool f32 = params->storage == LBM_STORAGE_F32;
-  c->launch_cfg[0] = f32 ? 1 : 0;
-  c->launch_cfg[1] = f32 ? 6 : 9;
-  c->launch_cfg[2] = f32 ? 7 : local ? 9 : 8;
-  c->launch_cfg_set = false;
   c->auto_lag = hmcsc::wave_auto_lag(sp);
-  c->choice_refused = false;
-  c->single_pass_zc = 0;
-  c->wave_cfg = 0;
-  c->wave_lag = hmcsc::kWaveLagDefault;
+  automatic_step(c);
   c->wave_spin = hmcsc::kWaveSpinDefault;
   c->wave_hold = -1;
   c->fault_seen = false;
@@ -738,8 +742,7 @@ lbm_status lbm_step(lbm_ctx *c, int n_steps) {
     // 16 blocks, or all blocks resident at once), which a stream limited to
     // some of the SMs refuses; nothing has been enqueued then, and the two
     // passes, which run anywhere, take over for good.
-    const bool own_choice = c->wave_cfg == 0 && c->single_pass_zc == 0 && !c->launch_cfg_set &&
-                            !c->choice_refused;
+    const bool own_choice = !c->step_set && !c->choice_refused;
     // Small lattices stay on the device for several steps; a reservoir change
     // takes effect at the end of a step, so the step it was made for is taken
     // on its own.
@@ -798,6 +801,7 @@ lbm_status lbm_set_single_pass(lbm_ctx *c, int planes) {
   if (planes > 0 && c->params.nx > hmcsc::kSinglePassMaxNx)
     return fail(c, LBM_EINVAL, "the single-pass step needs nx <= %d", hmcsc::kSinglePassMaxNx);
   c->single_pass_zc = planes;
+  c->step_set = true;
   return LBM_OK;
 }
 
@@ -812,6 +816,13 @@ lbm_status lbm_set_wavefront(lbm_ctx *c, int shape, int lag) {
     return fail(c, LBM_EINVAL, "wavefront lag too large for this lattice");
   c->wave_cfg = shape;
   c->wave_lag = lag;
+  c->step_set = true;
+  return LBM_OK;
+}
+
+lbm_status lbm_set_automatic_step(lbm_ctx *c) {
+  if (!c) return LBM_EINVAL;
+  automatic_step(c);
   return LBM_OK;
 }
 
@@ -1245,7 +1256,7 @@ lbm_status lbm_set_launch_config(lbm_ctx *c, int density_cfg, int even_cfg,
   c->launch_cfg[0] = density_cfg;
   c->launch_cfg[1] = even_cfg;
   c->launch_cfg[2] = odd_cfg;
-  c->launch_cfg_set = true;
+  c->step_set = true;
   return LBM_OK;
 }
 

@@ -40,6 +40,7 @@ ABI_SYMBOLS = (
     "lbm_set_geometry_per_component", "lbm_set_bc_velocity", "lbm_set_single_pass",
     "lbm_build_checked", "lbm_fault_word", "lbm_get_launch_config",
     "lbm_set_wavefront", "lbm_get_wavefront", "lbm_set_wavefront_limits",
+    "lbm_set_automatic_step",
 )
 LBM_DENSITY_CONFIGS, LBM_COLLIDE_CONFIGS = 3, 10
 SINGLE_PASS_MAX_NX = 256
@@ -100,6 +101,7 @@ def load(path: str | None = None):
         "lbm_set_bc": (ctypes.c_int, [vp, ctypes.c_int, ctypes.c_int, ctypes.c_double, ctypes.c_double]),
         "lbm_set_bc_velocity": (ctypes.c_int, [vp, ctypes.c_int, ctypes.c_int] + [ctypes.c_double] * 5),
         "lbm_step": (ctypes.c_int, [vp, ctypes.c_int]),
+        "lbm_set_automatic_step": (ctypes.c_int, [vp]),
         "lbm_set_single_pass": (ctypes.c_int, [vp, ctypes.c_int]),
         "lbm_set_wavefront": (ctypes.c_int, [vp, ctypes.c_int, ctypes.c_int]),
         "lbm_get_wavefront": (ctypes.c_int, [vp] + [ctypes.POINTER(ctypes.c_int)] * 2),
@@ -232,6 +234,10 @@ def lbm_fault_word(ctx, clear=True):
     v = ctypes.c_uint32(0)
     _check(ctx, load().lbm_fault_word(ctx, ctypes.byref(v), 1 if clear else 0))
     return int(v.value)
+
+
+def lbm_set_automatic_step(ctx):
+    return _check(ctx, load().lbm_set_automatic_step(ctx))
 
 
 def lbm_set_single_pass(ctx, planes):
@@ -443,23 +449,27 @@ class Lattice:
         """(density, even, odd) launch shapes in use."""
         return lbm_get_launch_config(self.ctx)
 
+    def set_automatic_step(self):
+        """The step of lbm_step's own choice again, as in a new lattice."""
+        lbm_set_automatic_step(self.ctx)
+
     def set_single_pass(self, planes):
         """Single-pass lbm_step with boxes of `planes` planes (0: two passes)."""
         lbm_set_single_pass(self.ctx, planes)
 
     def set_wavefront(self, shape, lag=0):
         """Wavefront lbm_step of tile shape `shape` (1: 32 x 4, 2: 32 x 2,
-        3: 32 x 8 nodes; 0: lbm_step's own choice) with densities `lag`
-        planes ahead (0: default); lbm_batch_step then also steps such lattices together in
-        one wavefront launch."""
+        3: 32 x 8 nodes; 0: two passes) with densities `lag` planes ahead
+        (0: default); lbm_batch_step then also steps such lattices together
+        in one wavefront launch."""
         lbm_set_wavefront(self.ctx, shape, lag)
 
     def wavefront(self):
-        """(shape, lag) of the wavefront step asked for (shape 0: none, the
-        step is lbm_step's own choice)."""
+        """(shape, lag) of the wavefront step asked for (shape 0: none)."""
         return lbm_get_wavefront(self.ctx)
 
     def set_launch_config(self, density_cfg=0, even_cfg=0, odd_cfg=0):
+        """Two passes in these launch shapes."""
         lbm_set_launch_config(self.ctx, density_cfg, even_cfg, odd_cfg)
 
     def autotune(self, table=None, single_pass=False):

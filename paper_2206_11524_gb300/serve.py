@@ -114,8 +114,8 @@ def make_requests(n_req=32, seed=2206, L_min=32, L_max=192, steps_min=1000,
     return reqs
 
 
-# Step form of the lattices the server and the baseline create: 0 = two
-# passes (the library's default step).  With a wavefront shape
+# Step form of the lattices the server and the baseline create: 0 = the
+# library's default step (batches: two passes).  With a wavefront shape
 # (lbm_set_wavefront) a batch steps in one persistent launch instead; on
 # this trace's lattices (32^3 .. 192^3: few tiles per plane, so the
 # dependency chain between groups leaves most blocks idle) that launch is
@@ -130,7 +130,8 @@ def _lattice_for(req: Request, storage: str, stream, wave=WAVE_BATCH):
     for face, (Lr, a, b) in req.reservoirs.items():
         lat.set_bc(face, Lr, a, b)
     lat.init_equilibrium(req.rho_a, req.rho_b)
-    lat.set_wavefront(wave)
+    if wave:
+        lat.set_wavefront(wave)
     return lat
 
 

@@ -232,12 +232,53 @@ static void undefined_state() {
   lbm_batch_graph_destroy(g);
 }
 
+// Asking for no wavefront, no single pass, or for launch shapes asks for the
+// two passes; lbm_set_automatic_step gives the choice back to the library.
+static void step_choice() {
+  const struct { int nx, ny, nz; const char *name; } own[] = {{32, 32, 32, "resident"}, {128, 128, 128, "wave"}};
+  for (const auto &o : own) {
+    Lattice l(o.nx, o.ny, o.nz);
+    int first[3], cfg[3], shape, lag;
+    CHECK(lbm_get_launch_config(l.ctx, &first[0], &first[1], &first[2]) == LBM_OK);
+    const auto takes = [&](const char *name) {
+      launched.clear();
+      CHECK(lbm_step(l.ctx, 1) == LBM_OK);
+      return launched.size() == 1 + !strcmp(name, "density") && launched[name] == 1;
+    };
+    CHECK(takes(o.name));
+    CHECK(lbm_set_wavefront(l.ctx, 0, 0) == LBM_OK);
+    CHECK(takes("density"));
+    CHECK(lbm_set_automatic_step(l.ctx) == LBM_OK);
+    CHECK(takes(o.name));
+    CHECK(lbm_set_single_pass(l.ctx, 3) == LBM_OK);
+    CHECK(takes("single_pass"));
+    CHECK(lbm_set_single_pass(l.ctx, 0) == LBM_OK);
+    CHECK(takes("density"));
+    CHECK(lbm_set_wavefront(l.ctx, 1, 5) == LBM_OK);
+    CHECK(takes("wave"));
+    CHECK(lbm_set_automatic_step(l.ctx) == LBM_OK);
+    CHECK(takes(o.name));
+    CHECK(lbm_get_wavefront(l.ctx, &shape, &lag) == LBM_OK);
+    CHECK(shape == 0 && lag == hmcsc::kWaveLagDefault);
+    CHECK(lbm_set_launch_config(l.ctx, 2, 3, 4) == LBM_OK);
+    CHECK(takes("density"));
+    CHECK(lbm_set_automatic_step(l.ctx) == LBM_OK);
+    CHECK(takes(o.name));
+    CHECK(lbm_get_launch_config(l.ctx, &cfg[0], &cfg[1], &cfg[2]) == LBM_OK);
+    CHECK(memcmp(first, cfg, sizeof cfg) == 0);
+    CHECK(lbm_set_launch_config(l.ctx, -1, 0, 0) == LBM_EINVAL);
+    CHECK(takes(o.name));
+  }
+  CHECK(lbm_set_automatic_step(nullptr) == LBM_EINVAL);
+}
+
 int main(int argc, char **argv) {
   const std::string name = argc > 1 ? argv[1] : "";
   if (name == "misaligned_destination") misaligned_destination();
   else if (name == "device_destination") device_destination();
   else if (name == "refused_choice") refused_choice();
   else if (name == "undefined_state") undefined_state();
+  else if (name == "step_choice") step_choice();
   else return std::printf("no check '%s'\n", name.c_str()), 2;
   if (failures == 0) std::printf("ok\n");
   return failures != 0;

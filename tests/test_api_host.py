@@ -31,7 +31,7 @@ def harness(tmp_path_factory):
 
 
 @pytest.mark.parametrize("check", ["misaligned_destination", "device_destination", "refused_choice",
-                                   "undefined_state"])
+                                   "undefined_state", "step_choice"])
 def test_host_side(harness, check):
     out = subprocess.run([harness, check], capture_output=True, text=True)
     assert out.returncode == 0 and out.stdout.strip() == "ok", out.stdout + out.stderr
