@@ -6,19 +6,20 @@ and optionally of the single-pass step.
 `tune(nx, ny, nz, storage)` times every shape on a scratch lattice of that
 size and storage (a synthetic gray medium with two-phase densities; the
 kernels' cost does not depend on the values) and returns the fastest.
-`TuneTable` keeps the winners in a JSON file keyed by GPU name, lattice size
-and storage, so a lattice of a known size is configured without timing
-(`apply(lattice)`).  The table lives at $HMCSC_TUNE_TABLE, else
+`TuneTable` keeps the winners in a JSON file keyed by GPU name, lattice size,
+storage and the kernels they were timed on, so a lattice of a known size is
+configured without timing (`apply(lattice)`).  The table lives at $HMCSC_TUNE_TABLE, else
 ~/.cache/hmcsc/launch_table.json.
 """
 from __future__ import annotations
 
+import functools
 import json
 import os
 
 import numpy as np
 
-from . import lbm
+from . import build, lbm
 
 
 def _default_path() -> str:
@@ -26,10 +27,15 @@ def _default_path() -> str:
         os.path.expanduser("~"), ".cache", "hmcsc", "launch_table.json")
 
 
+@functools.lru_cache(maxsize=None)
+def _kernels() -> str:
+    return build.kernel_hash()
+
+
 def _key(nx, ny, nz, storage) -> str:
     import torch
     name = torch.cuda.get_device_name(torch.cuda.current_device())
-    return f"{name}|{nx}x{ny}x{nz}|{storage}"
+    return f"{name}|{nx}x{ny}x{nz}|{storage}|{_kernels()}"
 
 
 class TuneTable:

@@ -6,7 +6,9 @@ statically so the library loads next to any PyTorch build.
 """
 from __future__ import annotations
 
+import hashlib
 import os
+import re
 import shutil
 import subprocess
 import sys
@@ -49,6 +51,17 @@ def _newest_input() -> float:
     paths.append(os.path.join(INCLUDE, "lbm.h"))
     paths.append(os.path.abspath(__file__))
     return max(os.path.getmtime(p) for p in paths)
+
+
+def kernel_hash() -> str:
+    """Hash of the kernels and their launchers, comments and blank lines left
+    out: what a timing of the library's launches is good for."""
+    h = hashlib.sha256()
+    for f in sorted(SOURCES + HEADERS):
+        with open(os.path.join(CSRC, f)) as fh:
+            code = re.sub(r"//[^\n]*", "", fh.read())
+        h.update("\n".join(l.rstrip() for l in code.splitlines() if l.strip()).encode())
+    return h.hexdigest()[:16]
 
 
 def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False,

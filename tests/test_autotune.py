@@ -1,0 +1,37 @@
+"""The tuner's table and its choice, on the CPU: entries belong to the kernels
+they were timed on, and a step replaces another only by the stated margin."""
+import json
+
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2206_11524_gb300 import autotune, build
+
+
+@pytest.fixture
+def gpu_name(monkeypatch):
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    monkeypatch.setattr(torch.cuda, "get_device_name", lambda _: "GPU")
+
+
+def test_an_entry_of_other_kernels_is_not_applied(tmp_path, monkeypatch, gpu_name):
+    path = tmp_path / "t.json"
+    # as written before entries named their kernels
+    path.write_text(json.dumps({"GPU|500x1x1|f32": {"config": [1, 6, 7, 0, 0, 0], "timings_ms": {}}}))
+    assert autotune.TuneTable(str(path)).get(500, 1, 1, "f32") is None
+    autotune.TuneTable(str(path)).put(500, 1, 1, "f32", (-1, -1, -1, 0, 0, 0), {})
+    assert autotune.TuneTable(str(path)).get(500, 1, 1, "f32") == (-1, -1, -1, 0, 0, 0)
+    monkeypatch.setattr(autotune, "_kernels", lambda: "other")
+    assert autotune.TuneTable(str(path)).get(500, 1, 1, "f32") is None
+
+
+def test_the_hash_follows_the_code_and_not_its_comments(tmp_path, monkeypatch):
+    for f in build.SOURCES + build.HEADERS:
+        (tmp_path / f).write_text("int a;  // one\n")
+    monkeypatch.setattr(build, "CSRC", str(tmp_path))
+    first = build.kernel_hash()
+    (tmp_path / build.HEADERS[0]).write_text("// more\n\nint a;\n")
+    assert build.kernel_hash() == first
+    (tmp_path / build.HEADERS[0]).write_text("int b;\n")
+    assert build.kernel_hash() != first
