@@ -124,6 +124,18 @@ def _single_pass_candidates(ny, nz, sms):
 WAVE_CANDIDATES = ((2, 4), (1, 4), (2, 5), (3, 4))
 
 
+def _choose(two, others, untuned, margin):
+    """Which step to keep from the times of a whole one: "two_pass" (`two`), a
+    key of `others` ((key, time) pairs), or "untuned", the library's own choice.
+    One of the others has to beat the two passes by `margin`, and the library's
+    choice the best of them all."""
+    best, ms, limit = "two_pass", two, two * (1.0 - margin)
+    for key, t in others:
+        if t < limit:
+            best, ms, limit = key, t, t
+    return "untuned" if untuned < ms * (1.0 - margin) else best
+
+
 def tune(nx, ny, nz, storage="f32", reps=10, single_pass=False, margin=0.03,
          wavefront=True):
     """Fastest (density, even, odd) launch shapes and all timings (ms),
@@ -174,16 +186,14 @@ def tune(nx, ny, nz, storage="f32", reps=10, single_pass=False, margin=0.03,
     best_sp, best_wave = 0, (0, 0)
     if single_pass or wavefront:
         lbm.lbm_set_launch_config(ctx, *cfg)
-        two = _step_ms(lat)
-        timings["two_pass_step"] = two
-        best_ms = two * (1.0 - margin)
+        timings["two_pass_step"] = _step_ms(lat)
+        others = []                        # ((single-pass depth, wavefront), ms)
         if wavefront:
             for shape, lag in WAVE_CANDIDATES:
                 lat.set_wavefront(shape, lag)
                 ms = _step_ms(lat)
                 timings[f"wavefront_{shape}_{lag}"] = ms
-                if ms < best_ms:
-                    best_wave, best_ms = (shape, lag), ms
+                others.append(((0, (shape, lag)), ms))
             lat.set_wavefront(0)
         if single_pass and nx <= lbm.SINGLE_PASS_MAX_NX:
             import torch
@@ -193,11 +203,13 @@ def tune(nx, ny, nz, storage="f32", reps=10, single_pass=False, margin=0.03,
                 lat.set_single_pass(planes)
                 ms = _step_ms(lat)
                 timings[f"single_pass_{planes}"] = ms
-                if ms < best_ms:
-                    best_sp, best_wave, best_ms = planes, (0, 0), ms
+                others.append(((planes, (0, 0)), ms))
             lat.set_single_pass(0)
-        if timings["untuned_step"] < best_ms * (1.0 - margin):
-            cfg, best_sp, best_wave = (-1, -1, -1), 0, (0, 0)
+        step = _choose(timings["two_pass_step"], others, timings["untuned_step"], margin)
+        if step == "untuned":
+            cfg = (-1, -1, -1)
+        elif step != "two_pass":
+            best_sp, best_wave = step
     lat.close()
     return cfg + (best_sp,) + best_wave, timings
 

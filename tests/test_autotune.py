@@ -35,3 +35,16 @@ def test_the_hash_follows_the_code_and_not_its_comments(tmp_path, monkeypatch):
     assert build.kernel_hash() == first
     (tmp_path / build.HEADERS[0]).write_text("int b;\n")
     assert build.kernel_hash() != first
+
+
+def test_each_step_has_to_win_by_the_margin_once():
+    wave, single = (0, (2, 4)), (8, (0, 0))
+    choose = autotune._choose
+    # 288^3: two passes 1718 us, the library's wavefront launch 1646, 4 % less
+    assert choose(1718.0, [(wave, 1700.0)], 1646.0, 0.03) == "untuned"
+    assert choose(100.0, [], 97.5, 0.03) == "two_pass"
+    assert choose(100.0, [(wave, 97.5)], 96.5, 0.03) == "untuned"   # the wavefront fell short
+    assert choose(100.0, [(wave, 90.0)], 88.0, 0.03) == wave        # 2 % on the best
+    assert choose(100.0, [(wave, 90.0)], 87.0, 0.03) == "untuned"
+    assert choose(100.0, [(wave, 90.0), (single, 89.0)], 95.0, 0.03) == single
+    assert choose(100.0, [(wave, 98.0), (single, 99.0)], 99.0, 0.03) == "two_pass"
