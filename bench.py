@@ -471,6 +471,14 @@ def large_domain_record(args, peak):
     return rec
 
 
+def _own_choice(launch, args):
+    """Is the timed step lbm_step's own choice of launch?  When neither the
+    launch shapes (given, or the tuner's; -1: it leaves the lattice alone) nor
+    another step are set."""
+    return (launch is None or launch[0] < 0) and not (
+        args.single_pass > 0 or args.wavefront or args.no_wavefront)
+
+
 def run_gpu(args, world, rank, local):
     import numpy as np
     import torch
@@ -509,6 +517,7 @@ def run_gpu(args, world, rank, local):
         from paper_2206_11524_gb300 import autotune
         table = autotune.TuneTable(os.path.join(tempfile.mkdtemp(), "launch_table.json"))
         launch = list(lat.autotune(table))
+    own = _own_choice(launch, args)
     launch = list(lat.launch_config())   # the shapes actually in use
 
     single = args.single_pass > 0
@@ -521,7 +530,7 @@ def run_gpu(args, world, rank, local):
     wave = list(lat.wavefront())          # the step in use (tuned or asked for)
     if wave[0] == 0 or single:
         wave = None
-    one_launch = single or wave is not None
+    one_launch = single or wave is not None or own
     for _ in range(args.warmup):
         if one_launch:
             lbm.lbm_step(ctx, 1)
@@ -545,7 +554,7 @@ def run_gpu(args, world, rank, local):
         e0, e1, e2 = ev[k]
         e0.record(stream)
         if one_launch:
-            lbm.lbm_step(ctx, 1)   # wavefront launch, or bulk sweep + seam launches
+            lbm.lbm_step(ctx, 1)   # wavefront launch, bulk sweep + seam launches, or its choice
         else:
             lbm.lbm_density(ctx)
         e1.record(stream)
@@ -596,6 +605,14 @@ def run_gpu(args, world, rank, local):
         bytes_launch = bytes_collide * N
         achieved = bytes_launch / (ms_density / 1e3) / 1e9
         traffic_bpn = _profiled_traffic("wave") if storage == "f32" else None
+        step_gbs = bytes_launch / (ms_max / K / 1e3) / 1e9
+    elif own:
+        # whole step in the launch lbm_step picks for the size: the populations
+        # through DRAM once at least
+        kernel_name = "lbm_step (the library's choice)"
+        bytes_launch = bytes_collide * N
+        achieved = bytes_launch / (ms_density / 1e3) / 1e9
+        traffic_bpn = None
         step_gbs = bytes_launch / (ms_max / K / 1e3) / 1e9
     elif single:
         # whole single-pass step: every node 320 B as in the fused pass, and
@@ -665,6 +682,7 @@ def run_gpu(args, world, rank, local):
                      "traffic": (traffic_bpn * N if traffic_bpn else None)},
         "kernels_ms": ({"wavefront_step": ms_density} if wave is not None else
                        {"single_pass_step": ms_density} if single else
+                       {"own_choice_step": ms_density} if own else
                        {"density": ms_density, "collide_stream": ms_collide}),
         "step_hbm_gbs": step_gbs,
         "step_frac": step_gbs / peak,
@@ -673,8 +691,8 @@ def run_gpu(args, world, rank, local):
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d / K,
                 "d2h_bytes_per_step": d2h / K},
         # density pass + fused pass per step, bulk sweep + 2 seam launches,
-        # or one wavefront launch
-        "gpu_launches": (1 if wave is not None else 3 if single else 2) * K,
+        # one wavefront launch, or (the library's choice) one launch at least
+        "gpu_launches": (1 if wave is not None or own else 3 if single else 2) * K,
         "clocks": clk,
         "cpu_baseline": cpu,
         "large_domain": large,

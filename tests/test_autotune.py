@@ -1,5 +1,6 @@
 """The tuner's table and its choice, on the CPU: entries belong to the kernels
 they were timed on, and a step replaces another only by the stated margin."""
+import argparse
 import json
 
 import pytest
@@ -48,3 +49,17 @@ def test_each_step_has_to_win_by_the_margin_once():
     assert choose(100.0, [(wave, 90.0)], 87.0, 0.03) == "untuned"
     assert choose(100.0, [(wave, 90.0), (single, 89.0)], 95.0, 0.03) == single
     assert choose(100.0, [(wave, 98.0), (single, 99.0)], 99.0, 0.03) == "two_pass"
+
+
+def test_bench_times_the_step_that_runs():
+    """Where the tuner leaves the lattice alone the benchmark times lbm_step,
+    not the halves of a two-pass step."""
+    import bench
+
+    def own(launch, **set_):
+        args = {"single_pass": 0, "wavefront": "", "no_wavefront": False} | set_
+        return bench._own_choice(launch, argparse.Namespace(**args))
+    assert own([-1, -1, -1, 0, 0, 0]) and own(None)
+    assert not own([1, 6, 7, 0, 0, 0]) and not own([1, 6, 7])
+    assert not own([-1, -1, -1, 0, 0, 0], no_wavefront=True)
+    assert not own([-1, -1, -1, 0, 0, 0], wavefront="2,4") and not own(None, single_pass=4)
