@@ -96,16 +96,29 @@ void collide_any(const StepParams &p, const Workspace &w, int cfg, cudaStream_t 
     default: collide_cfg<PARITY, 0>(p, w, s);
   }
 }
+// A grid has at most 65,535 blocks along y and z.  Where a shape needs more for
+// a lattice, one takes its place that fits every lattice the library accepts
+// (ny <= 262,140, nz <= 131,070): 4 x 2 nodes for the density pass, 8 rows and
+// runs of planes for the fused pass (a prefetching shape's runs are 16 planes
+// long from 1,824 x 16 planes on, so only its rows count).
+constexpr int kGridYZ = 65535, kDensityTall = 0, kCollideTall = 6;
+bool grid_fits(const StepParams &p, int by, int bz) {
+  return (p.ny + by - 1) / by <= kGridYZ && (p.nz + bz - 1) / bz <= kGridYZ;
+}
 }  // namespace
 
 cudaError_t HMCSC_NAME(launch_density)(const StepParams &p, const Workspace &w,
                                        int parity, int cfg, cudaStream_t s) {
+  const Shape S = density_shape(cfg);
+  if (!grid_fits(p, S.by, S.bz)) cfg = kDensityTall;
   if (parity == 0) density_any<0>(p, w, cfg, s); else density_any<1>(p, w, cfg, s);
   return cudaGetLastError();
 }
 
 cudaError_t HMCSC_NAME(launch_collide)(const StepParams &p, const Workspace &w,
                                        int parity, int cfg, cudaStream_t s) {
+  const Shape S = collide_shape(parity, storage_local(kST), cfg);
+  if (!grid_fits(p, S.by, cfg >= kCollidePipeFirst ? 16 : S.bz)) cfg = kCollideTall;
   if (parity == 0) collide_any<0>(p, w, cfg, s); else collide_any<1>(p, w, cfg, s);
   return cudaGetLastError();
 }
