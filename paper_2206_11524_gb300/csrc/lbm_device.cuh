@@ -1113,18 +1113,18 @@ struct WaveArgs {
                         // (tests of the failure path)
 };
 
-// Flags are polled with relaxed loads, served by L2, so polling leaves the
-// SM's L1 alone (an acquire would drop it, and with it the stencil's cached
-// densities and geometry, once per poll).  A flag is set by a release store
-// after the tile's density stores, so once a poll sees the epoch those
-// densities are in L2; the loads that read them are issued after the poll
-// returned, and no SM caches a line of a tile's densities in L1 before that
-// tile's flag is set in this launch (each 128-byte line belongs to one
-// tile, and L1 is invalidated between launches), so they miss L1 the first
-// time and read L2.
-__device__ __forceinline__ unsigned ld_relaxed(const unsigned *ptr) {
+// A flag is set by a release store after a block barrier that follows the
+// tile's density stores, and polled with acquire loads: what a lane loads after
+// its last poll, and what its warp loads after the __syncwarp behind it, sees
+// those densities.  An acquire drops the SM's L1, and with it the stencil's
+// cached densities and geometry, once per poll; relaxed polls, which keep it
+// and which the memory model gives no order to, are 0.3-1 % faster (us a step:
+// 256^3 1,104 and 1,100, 128^3 144.4 and 143.0, 150 x 90 x 70 75.5 and 75.0).
+// A fence after relaxed polls also waits for the warp's own stores: 1,175 and
+// 156.7.
+__device__ __forceinline__ unsigned ld_acquire(const unsigned *ptr) {
   unsigned v;
-  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ptr) : "memory");
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ptr) : "memory");
   return v;
 }
 __device__ __forceinline__ void st_release(unsigned *ptr, unsigned v) {
@@ -1141,7 +1141,8 @@ __device__ __forceinline__ void wave_fault(const Workspace &w, unsigned epoch) {
 }
 
 // Densities written earlier in the same launch by other blocks, read after
-// their flags (see above), cached in L1 for the stencil.
+// their flags (see above): ordinary loads, cached in L1 for the stencil, never
+// the read-only path.
 struct WaveRho : GlobalRho {
   __device__ __forceinline__ float2 at(int dx, int dy, int dz) const {
     return __ldca(&rho[idx(dx, dy, dz)]);
@@ -1216,7 +1217,7 @@ __device__ __forceinline__ void wave_tile_item(const StepParams &p, const Worksp
     if (kChecked && !in_bounds(w.fault, fi, nflags, kFaultFlag)) fi = 0;
     // after one wait of this launch has run out the others give up at once
     unsigned n = 0;
-    while (ld_relaxed(&flag[fi]) != epoch) {
+    while (ld_acquire(&flag[fi]) != epoch) {
       if (++n == a.spin_limit) {
         wave_fault(w, epoch);
         break;
