@@ -47,7 +47,7 @@ __host__ __device__ constexpr int wclass(int i) {
 }
 
 // Half offsets are kept scaled by 2^14 (see above).
-constexpr float kHalfScale = 16384.0f, kHalfUnscale = 1.0f / 16384.0f;
+constexpr float kHalfScale = 16384.0f;
 
 // Packed arithmetic on the pair (sigma = 1, 2): one instruction does both
 // components, each rounded as the scalar operation would be (add.f32x2,
@@ -248,7 +248,7 @@ struct Workspace {
   float *ns2;        // [ntiles * 32] n_s,2, or nullptr: one fraction for both
   float *ads2;       // [ntiles * 32] G_ads,2 * n_s,2, or nullptr
   float *stage;      // [6][nlin] linear (x fastest) staging for host transfers
-  double *red;       // [kRedBlocks][kRedK] partial sums + [kRedK] result
+  double *red;       // [kRedBlocks][kRedK] partial sums
   unsigned *fault;   // bits of the accesses that were out of range in
                      // bounds-checked builds, and of wavefront waits that
                      // ran out in any build (FaultBits)

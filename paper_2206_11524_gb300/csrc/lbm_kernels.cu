@@ -145,7 +145,7 @@ size_t workspace_bytes(long long nx, long long ny, long long nz, int storage,
   size_t o_ns = take(sizeof(float) * nt);
   size_t o_ads = take(sizeof(float) * nt);
   size_t o_stage = take(sizeof(float) * 6 * (size_t)t.nlin);
-  size_t o_red = take(sizeof(double) * (kRedBlocks + 1) * kRedK);
+  size_t o_red = take(sizeof(double) * kRedBlocks * kRedK);
   size_t o_ns2 = take(per_component ? sizeof(float) * nt : 0);
   size_t o_ads2 = take(per_component ? sizeof(float) * nt : 0);
   size_t o_fault = take(sizeof(unsigned));
