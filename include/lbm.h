@@ -176,9 +176,11 @@ LBM_API lbm_status lbm_set_bc_velocity(lbm_ctx *ctx, int face, int layers,
  * same results bit for bit: a small lattice (up to 4,608 x-tiles: nx / 32,
  * rounded up, times ny nz) up to 256 steps per launch, a larger float32 lattice
  * whose planes in flight stay in L2 the wavefront launch with a lag of the
- * library's choice; all waits are bounded like the wavefront's, and
- * where such a launch is refused (a stream that may use only some of the SMs)
- * the two passes run instead.  n_steps = 0 is a no-op.  EINTERNAL (and
+ * library's choice.  These launches are made for one lattice at a time: where
+ * many small lattices step at once, lbm_batch_step, or two passes on streams of
+ * their own (lbm_set_wavefront with shape 0), does more steps in all.  All
+ * waits are bounded like the wavefront's, and where such a launch is refused
+ * (a stream that may use only some of the SMs) the two passes run instead.  n_steps = 0 is a no-op.  EINTERNAL (and
  * nothing enqueued) when a device fault was reported for the current state:
  * by a synchronising call (below), or by a launch that already ran, through
  * a host-mapped word the kernel sets (no stream wait). */
@@ -189,9 +191,9 @@ LBM_API lbm_status lbm_step(lbm_ctx *ctx, int n_steps);
  * EINVAL: NULL ctx. */
 LBM_API lbm_status lbm_set_automatic_step(lbm_ctx *ctx);
 
-/* Single-pass stepping for lbm_step (planes > 0; 0 = two passes): each step reads every population once.  The lattice is cut into
- * boxes of full x-rows, 8 rows by `planes` planes; one launch marches every
- * box along z, computing the densities of the next plane into shared memory
+/* Single-pass stepping for lbm_step (planes > 0; 0 = two passes): each step
+ * reads every population once.  The lattice is cut into boxes of full x-rows, 8
+ * rows by `planes` planes; one launch marches every box along z, computing the densities of the next plane into shared memory
  * and colliding the current plane's inner rows with them; the last row and
  * plane of each box (its seams, whose populations no other box may see
  * updated) are then updated by a second launch.  Results are bit-identical

@@ -508,11 +508,11 @@ __host__ __device__ constexpr Shape density_shape(int cfg) {
 // Shapes of the prefetching fused pass (k_collide_pipe): block 32 x by,
 // blocks per SM.  On the 256^3 electrode (us, even / odd step; 168 and 176
 // bytes a node at the copy rate of 6690 GB/s are 421 and 441): half offsets
-// 519/586 in shape 6, 430/520 in shapes 9/8 (scalar code, 8-byte copies and
-// no stencil ring on even steps: 606/737); local half offsets 693/728 in
-// shape 6, 455/553 in shape 9 (726/810), and 547 on even steps without its
-// streaming stores; float32 (320 bytes: 803) 774/885 in shape 6, 816/881 in
-// shape 7 (837/967), 778/985 in shape 9.  Even steps are bound by HBM.  Odd
+// 519/586 in shape 6, 430/520 in shapes 9/8 (in scalar operations with a copy
+// per population 606/737); local half offsets 693/728 in shape 6, 455/553 in
+// shape 9 (scalar 726/810; without its streaming stores 547 on even steps);
+// float32 (320 bytes: 803) 774/885 in shape 6, 816/881 in shape 7 (scalar
+// 837/967), 778/985 in shape 9.  Even steps are bound by HBM.  Odd
 // ones store rows shifted by a node, which leave part of a sector at either
 // end, and keep 18 addresses: they issue 753-788 instructions a node, 61 % of
 // the slots, and the local storages take 168 registers.  Staging the stencil
@@ -1084,9 +1084,8 @@ __global__ void k_init_equilibrium(StepParams p, Workspace w,
 // stays race-free: the collision of node n touches only the slots holding
 // n's own populations, whose density part has finished reading them before
 // n's flag is set.
-// One float32 step of 256^3 takes 1,103 us (1,156 with scalar arithmetic and
-// rows not uniform) and moves 335 bytes a node, against 1,210 us and 476 in
-// two passes.  What bounds it is the chain of each item -- copies from DRAM,
+// One float32 step of 256^3 takes 1,106 us and moves 335 bytes a node, against
+// 1,210 us and 476 in two passes (in scalar operations 1,156).  What bounds it is the chain of each item -- copies from DRAM,
 // flags, stencil from L2 -- at 16 warps per SM: fewer instructions (divisions
 // as multiplications, copies in chunks) did not shorten it, nor did
 // publishing before the collision's stores.

@@ -52,10 +52,11 @@ constexpr float kHalfScale = 16384.0f;
 // Packed arithmetic on the pair (sigma = 1, 2): one instruction does both
 // components, each rounded as the scalar operation would be (add.f32x2,
 // mul.f32x2, fma.f32x2).  Both components take the same steps everywhere on
-// the path, and the 16-bit fused passes were bound by instruction issue
-// (1,115-1,289 instructions a node in scalar form, 691-788 now, row copies
-// included), so the pairs stay pairs from the load to the store.  A subtraction is a fused multiply-add with
-// -1, which rounds once like the subtraction it stands for.
+// the path, and the 16-bit fused passes are bound by instruction issue, so the
+// pairs stay pairs from the load to the store: 691 (even) and 788 (odd)
+// instructions a node in local half offsets, against 1,115 and 1,289 in scalar
+// operations with a copy per population.  A subtraction is a fused
+// multiply-add with -1, which rounds once like the subtraction it stands for.
 // A packed product that feeds a packed sum is fused with it by the assembler
 // (measured: mul2 into add2 rounds once, .rn or not), so where both roundings
 // matter one of the two operations is written scalar.
@@ -304,17 +305,22 @@ constexpr int kRedBlocks = 2 * kSms;
 // Lag.  8 blocks per SM hold 1,216 items at a time, and a collision needs the
 // densities of two groups of tiles fewer than lag back, so the launch starves
 // unless (lag - 2) groups are well over what is in flight; every plane more
-// costs L2.  Measured for (lag - 2) x tiles per plane, us a step: 128^3 1,536
-// 245, 2,048 143, 2,560 144, 4,096 157; 192^3 1,728 586, 2,304 455, 2,880 474;
-// 224^3 1,568 1,141, 2,352 726, 3,136 772; 256^3 1,024 2,581, 2,048 1,103,
-// 3,072 1,165.  Hence the least lag that reaches 2,040.
+// costs L2.  Measured for (lag - 2) x tiles per plane, us a step: 128^3 1,792
+// 175, 2,048 144, 2,304 145; 192^3 1,728 590, 2,304 458, 2,880 478; 256^3 1,024
+// 2,594, 2,048 1,106, 3,072 1,175; 160 x 204 x 160 1,530 560, 2,040 343, 2,550
+// 345; 128 x 102 x 128 1,836 134, 2,040 117, 2,244 118; 97 x 131 x 61 1,848 81,
+// 2,112 74; 64 x 64 x 500 1,536 255, 1,920 147, 2,048 141, 2,112 141; 64 x 68 x
+// 170 1,496 102, 1,972 60, 2,040 59.  Hence the least lag that reaches 2,040.
 //
-// Where it wins (two passes, wavefront, us a step): 96^3 73.2, 68.4; 128^3
-// 168, 143; 150 x 90 x 70 81, 75; 160^3 319, 268; 192^3 524, 455; 224^3 822,
-// 726; 400 x 100 x 300 885, 792; 256^3 1,210, 1,103; 288^3 1,718, 1,646
+// Where it wins (two passes, wavefront, us a step): 96^3 73.0, 68.4; 128^3
+// 168, 144; 150 x 90 x 70 81, 75; 160^3 320, 270; 192^3 525, 458; 224^3 821,
+// 731; 400 x 100 x 300 886, 798; 256^3 1,210, 1,106; 288^3 1,720, 1,657
 // (76 MB of planes in flight); 320^3 2,347, 2,362 (93 MB); 512 x 512 x 100
 // 1,878, 1,982 -- while lag + 2 planes stay in L2.  A launch runs nz + lag
-// groups, so short lattices lose: nz of five lags at least.  The 16-bit
+// groups, so short lattices lose: nz of five lags at least.  Columns of few
+// tiles and long lags: 64 x 64 x 500 (34) 165, 141; 32 x 16 x 2000 (257) 83,
+// 75; 1 x 1 x 20000 (2,042) 84, 68; close to five lags both are alike, 64 x 64
+// x 170 57, 56, 32 x 16 x 1300 52, 53, 8 x 40 x 1000 (104) 75, 78.  The 16-bit
 // storages stay with two passes, whose stencil comes from shared memory
 // (128^3 half offsets 107, 132).
 inline int wave_auto_lag(const StepParams &p) {

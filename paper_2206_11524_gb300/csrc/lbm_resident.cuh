@@ -1,23 +1,31 @@
 // lbm_resident.cuh -- several time steps of a small lattice in one launch.
 //
-// A small lattice is bound by latency: the two launches of a step took 8 us
+// A small lattice is bound by latency: the two launches of a step take 8 us
 // for 500 nodes, whose arithmetic takes well under one.  Here the blocks stay
 // for all the steps of the launch: per step a warp sums the densities of its
 // x-tiles, meets a barrier of the whole grid, collides and streams them, and
 // meets it again.  The sums and collisions are those of the two passes, so
-// the results are bit-identical.
+// the results are bit-identical.  (Times: us a step, float32, two passes and
+// here.)
 //
 //   k_cluster   up to kClusterTiles x-tiles: one tile per warp, one cluster,
 //               the populations and densities in its shared memory for the
 //               whole launch, neighbours read and written across the
-//               cluster, the hardware's cluster barrier.  500 x 1 x 1 nodes:
-//               8.2 -> 1.3 us a step, 50 x 50: 8.2 -> 1.6, 64 x 64: 10.3 ->
-//               1.8 (float32; state in L2 instead: 4.1 us).
+//               cluster, the hardware's cluster barrier.  500 x 1 x 1 nodes
+//               8.2, 1.3 (state in L2 instead: 4.1), 50 x 50 9.4, 1.8,
+//               64 x 64 9.7, 1.8.
 //   k_resident  up to kResidentTiles: the state in the workspace (L2), a
 //               counter in the workspace as barrier, cooperative.  32 x 16 x
-//               16: 10.3 -> 5.4 us a step, 32^3: 10.3 -> 5.7, 48^3: 15.4 ->
-//               13.6; beyond that the two passes win (64^3: 21.5 against
-//               21.8, 80^3: 40 against 47).
+//               16 10.3, 4.4, 32^3 10.3, 5.5, 48^3 14.4, 13.3; beyond that the
+//               two passes win (64^3 21.5, 21.8, 80^3 39.5, 47).
+//
+// k_resident is for one lattice at a time: its blocks of eight warps at 204-254
+// registers leave no room for another's on an SM, so lattices of more than some
+// 600 tiles on streams of their own take turns, where the passes of several
+// overlap (eight lattices, us per lattice step, here and in two passes: 32^3
+// 5.6, 2.9, 40^3 10.8, 7.3, 48^3 13.6, 11.4, 200 x 200 x 1 7.4, 3.0).  Held to
+// 128 registers two fit (32^3 3.8, 48^3 8.9), but one alone then takes 7 %
+// longer in float32 and 15-25 % in the local storages.
 #pragma once
 #include "lbm_device.cuh"
 

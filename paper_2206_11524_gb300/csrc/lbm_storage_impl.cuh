@@ -251,7 +251,7 @@ cudaError_t resident_launch(const StepParams &p, const Workspace &w, int parity,
     cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev);
   });
   if (sms[dev] < 1) return cudaErrorInvalidDevice;
-  // few warps a block while that leaves SMs free (32 x 16 x 16: 4.6 us a step
+  // few warps a block while that leaves SMs free (32 x 16 x 16: 4.4 us a step
   // in 128 blocks of two warps, 5.4 in 32 of eight)
   int warps = 1;
   while (warps < kResidentWarps && p.ntiles > (long long)warps * sms[dev]) warps *= 2;
